@@ -185,7 +185,7 @@ def sersic_draw(rng, H, W, bright):
     """A galaxy as in the survey-like configuration: n ~ U[0.5, 6], r_e log-uniform, q ~ U[0.2, 1], flux over
     three decades.  bright: a resolved, bright one, whose fit ends at a well-determined minimum."""
     side = min(H, W)
-    n, q = (rng.uniform(0.8, 1.7), rng.uniform(0.3, 0.7)) if bright else (rng.uniform(0.5, 6.0), rng.uniform(0.2, 1.0))
+    n, q = (rng.uniform(0.8, 1.7), rng.uniform(0.5, 0.75)) if bright else (rng.uniform(0.5, 6.0), rng.uniform(0.2, 1.0))
     a, b = (6.0, max(8.0, min(30.0, 0.12 * side))) if bright else (2.0, min(40.0, 0.2 * side))
     re = math.exp(rng.uniform(math.log(a), math.log(b)))
     flux = math.exp(rng.uniform(math.log(1e5 if bright else 1e2), math.log(1e6 if bright else 1e5)))
