@@ -2098,7 +2098,7 @@ gf_status check_cnn_batch(int batch)
 
 // a guess call's tables in its workspace: H, W (int), offsets (int64), lo, hi
 struct GuessLayout {
-    size_t H, W, off, lo, hi, e2, total;
+    size_t H, W, off, lo, hi, total;
 };
 
 GuessLayout guess_layout(int count)
@@ -2115,7 +2115,6 @@ GuessLayout guess_layout(int count)
     g.off = take(sizeof(long long) * (size_t)count);
     g.lo = take(sizeof(double) * kGuessSlots);
     g.hi = take(sizeof(double) * kGuessSlots);
-    g.e2 = take(sizeof(double));  // the Sersic flux factor at n = 2
     g.total = o;
     return g;
 }
@@ -2256,16 +2255,17 @@ gf_status gf_default_guess(const gf_batch* b, const float* img, double* params, 
     std::vector<long long> off(count);
     size_t smem = 0;
     long long run = 0;
-    int max_npx = 0;
+    int max_npx = 0, max_rows = 0;
     for (int i = 0; i < count; ++i) {
         if (H[i] < 1 || W[i] < 1 || (long long)H[i] * W[i] > (1LL << 30))
             return fail(GF_EINVAL, "stamp size out of range");
         smem = std::max(smem, default_guess_smem(H[i], W[i]));
         max_npx = (int)std::min<long long>(std::max<long long>(max_npx, (long long)H[i] * W[i]), INT_MAX);
+        max_rows = std::max(max_rows, H[i]);
         off[i] = b->pix_off ? (long long)b->pix_off[i] : run;
         run += (long long)H[i] * W[i];
     }
-    if (smem > 64 * 1024) return fail(GF_EINVAL, "default guess: stamp ring longer than 8192 pixels");
+    if (smem > sizeof(unsigned) * 8192) return fail(GF_EINVAL, "default guess: stamp ring longer than 8192 pixels");
     const GuessLayout g = guess_layout(count);
     gf_status r = check_ws(ws, ws_bytes, g.total);
     if (r != GF_OK) return r;
@@ -2276,7 +2276,7 @@ gf_status gf_default_guess(const gf_batch* b, const float* img, double* params, 
     memcpy(blob.data() + g.off, off.data(), sizeof(long long) * count);
     if ((r = upload(ws, blob, s)) != GF_OK) return r;
     GF_CUDA(default_guess(count, at<int>(ws, g.H), at<int>(ws, g.W), at<long long>(ws, g.off), img,
-                          params, kGuessSlots, smem, max_npx, at<double>(ws, g.e2), s));
+                          params, kGuessSlots, smem, max_npx, max_rows, s));
     return GF_OK;
 }
 
