@@ -126,10 +126,13 @@ typedef enum {
 } gf_comp_kind;
 
 typedef enum {
-    GF_CONV_AUTO = 0,   /* direct for P < GF_AUTO_FFT_PSF, else FFT.  (For extended
-                           grids up to 160 x 160 the FFT is one CTA per transform and
-                           overtakes the direct sum from about P = 15 on 64x64 and
-                           96x96 stamps, P = 33 on 32x32: name GF_CONV_FFT there.) */
+    GF_CONV_AUTO = 0,   /* direct for P < GF_AUTO_FFT_PSF, else FFT.  The batched calls
+                           (gf_eval_batch, gf_eval_batch_dev, gf_lm_fit_batch,
+                           gf_lm_fit_multistart) take P from 23 to 39 through the FFT's
+                           one-CTA transform instead, in overlapping tiles, for stamps of
+                           any sizes.  (Stamps of one size whose extended grid is at most
+                           160 x 160 are one transform each under GF_CONV_FFT: name it
+                           there.) */
     GF_CONV_DIRECT = 1, /* tiled direct sum, PSF and halo tile in shared memory */
     GF_CONV_FFT = 2,    /* shared-memory mixed-radix FFT, 2^a 3^b 5^c sizes up to 4096;
                            the stamps of one call must share H and W.  Extended grids

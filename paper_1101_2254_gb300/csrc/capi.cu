@@ -121,6 +121,29 @@ int comp_slots(int kind)
     }
 }
 
+// The batched calls' convolution under GF_CONV_AUTO for PSF sides in
+// [TILED_MIN_PSF, GF_AUTO_FFT_PSF): overlap-save tiles through the one-CTA
+// transform (conv_fft.cu), for stamps of any sizes.  Not a value that a caller
+// may name.  The direct sum costs P^2 FMAs an output, a tile's transforms the
+// same for every P.  Convolution of one evaluation, PSF spectra included (us,
+// direct / tiled):
+//   400 stamps of 32-256 px   P 21: 187 / 130   25: 236 / 134   33: 424 / 135   39: 676 / 199
+//   400 stamps of 48-64 px    P 21:  53 / 58    25:  67 / 57    33:  98 / 68    39: 176 / 85
+// and a fit makes the spectra once.  The line depends on P alone, so that a
+// stamp's result does not depend on the batch around it; single-stamp calls,
+// where the set-up's launches count, keep the direct sum.
+constexpr int CONV_TILED = 100;
+constexpr int TILED_MIN_PSF = 23;
+
+// d as a batched call resolves it (d is checked)
+gf_desc batch_desc(const gf_desc* d)
+{
+    gf_desc e = *d;
+    if (e.conv_method == GF_CONV_AUTO && e.psf_size >= TILED_MIN_PSF && e.psf_size < GF_AUTO_FFT_PSF)
+        e.conv_method = CONV_TILED;
+    return e;
+}
+
 int resolve_method(const gf_desc* d)
 {
     if (d->conv_method == GF_CONV_AUTO)
@@ -495,9 +518,10 @@ struct Plan {
     Layout L;
     std::vector<StampInfo> st;
     std::vector<int> pre;  // 4 * (count + 1): model, os, conv, red
-    int method;            // GF_CONV_DIRECT, GF_CONV_FFT or GF_CONV_DFT_TC
-    int Nx, Ny, cpc;       // FFT geometry (method FFT)
+    int method;            // GF_CONV_DIRECT, GF_CONV_FFT, CONV_TILED or GF_CONV_DFT_TC
+    int Nx = 0, Ny = 0, cpc = 0;  // FFT geometry (methods FFT and tiled)
     int small = 0;         // FFT: one CTA per transform (Nx, Ny in 32 x {3, 4, 5})
+    int toy = 0, tox = 0;  // small: outputs of a tile (the stamp's own size, method FFT)
     DftFactor fx, fy;      // DFT geometry (method DFT_TC)
 };
 
@@ -552,6 +576,29 @@ void plan_batch(const gf_desc* d, const Structure& S, int count, const int* H, c
         max_wb = std::max<long long>(max_wb, nwb);
         max_red = std::max(max_red, pr[b + 1] - pr[b]);
     }
+    pl->method = resolve_method(d);
+    if (pl->method == GF_CONV_FFT) {
+        // grids up to 160 x 160: padded to 32 M and transformed one CTA each,
+        // the spectrum kept in shared memory (no spectrum scratch)
+        const StampInfo& s0 = pl->st[0];
+        pl->Nx = fft_small_len(s0.We);
+        pl->Ny = fft_small_len(s0.He);
+        pl->small = pl->Nx > 0 && pl->Ny > 0;
+        pl->toy = s0.H;
+        pl->tox = s0.W;
+    }
+    if (pl->method == CONV_TILED) {
+        pl->Nx = pl->Ny = fft_tile_len(P);
+        pl->small = 1;
+        pl->toy = fft_tile_toy(P);
+        pl->tox = fft_tile_tox(P);
+    }
+    if (pl->small)  // the convolution's work items are the transform's tiles
+        for (int b = 0; b < count; ++b) {
+            const StampInfo& s = pl->st[b];
+            pc[b + 1] = pc[b] + ((s.H + pl->toy - 1) / pl->toy) * ((s.W + pl->tox - 1) / pl->tox);
+            pc32[b + 1] = 0;
+        }
     Layout& L = pl->L;
     memset(&L, 0, sizeof(L));
     L.max_red = max_red;
@@ -638,20 +685,13 @@ void plan_batch(const gf_desc* d, const Structure& S, int count, const int* H, c
         L.wl_blk = o;
         o += al(sizeof(int) * (size_t)worklist_blocks(count) * (1 + WK_KINDS));
     }
-    pl->method = resolve_method(d);
-    if (pl->method == GF_CONV_FFT) {
+    if (pl->method == GF_CONV_FFT || pl->method == CONV_TILED) {
         const StampInfo& s0 = pl->st[0];
-        pl->Nx = fft_len(s0.We, true);
-        pl->Ny = fft_len(s0.He, false);
-        pl->cpc = choose_cpc(pl->Ny);
-        // grids up to 160 x 160: padded to 32 M and transformed one CTA each,
-        // the spectrum kept in shared memory (no spectrum scratch)
-        const int sx = fft_small_len(s0.We), sy = fft_small_len(s0.He);
-        pl->small = sx > 0 && sy > 0;
-        if (pl->small) {
-            pl->Nx = sx;
-            pl->Ny = sy;
+        if (!pl->small) {
+            pl->Nx = fft_len(s0.We, true);
+            pl->Ny = fft_len(s0.He, false);
         }
+        pl->cpc = choose_cpc(pl->Ny);
         const size_t Kx = pl->Nx / 2 + 1;
         L.tw_x = o;
         o += al(sizeof(float2) * pl->Nx);
@@ -660,7 +700,7 @@ void plan_batch(const gf_desc* d, const Structure& S, int count, const int* H, c
         L.hhat = o;
         o += al(sizeof(float2) * (size_t)count * pl->Ny * Kx);
         L.psfgrid = o;
-        o += al(sizeof(float) * (size_t)count * pl->Ny * pl->Nx);
+        if (pl->method == GF_CONV_FFT) o += al(sizeof(float) * (size_t)count * pl->Ny * pl->Nx);
         const size_t spec_rows = pl->small ? 0 : (size_t)s0.He * Kx;
         if (need & (NEED_JAC | NEED_LM)) {
             L.spec_jac = o;
@@ -814,6 +854,9 @@ FFTArgs fft_args(void* ws, const Plan& pl)
     f.Ny = pl.Ny;
     f.cpc = pl.cpc;
     f.small = pl.small;
+    f.toy = pl.toy;
+    f.tox = pl.tox;
+    f.one_tile = pl.method == GF_CONV_FFT;
     f.px = make_fft_plan(pl.Nx);
     f.py = make_fft_plan(pl.Ny);
     f.tw_x = at<float2>(ws, pl.L.tw_x);
@@ -1017,7 +1060,7 @@ gf_status setup_conv(void* ws, const Plan& pl, const float* psf, cudaStream_t s)
         ProfScope ps(PROF_CONV, s);
         return setup_conv_dft(ws, pl, psf, s);
     }
-    if (pl.method != GF_CONV_FFT) return GF_OK;
+    if (pl.method == GF_CONV_DIRECT) return GF_OK;
     ProfScope ps(PROF_CONV, s);
     const FFTArgs f = fft_args(ws, pl);
     GF_CUDA(launch_fft_twiddles(f, s));
@@ -1320,6 +1363,8 @@ size_t gf_workspace_size_eval_batch(const gf_desc* d, const gf_batch* b)
 {
     if (!b || b->count < 1 || !b->H || !b->W) return 0;
     if (check_structure(d) != GF_OK) return 0;
+    const gf_desc db = batch_desc(d);
+    d = &db;
     for (int i = 0; i < b->count; ++i)
         if (check_stamp(d, b->H[i], b->W[i]) != GF_OK) return 0;
     if (check_fft(d, b->count, b->H, b->W) != GF_OK) return 0;
@@ -1334,6 +1379,8 @@ size_t gf_workspace_size_batch(const gf_desc* d, const gf_batch* b, const uint8_
 {
     if (!b || b->count < 1 || !b->H || !b->W) return 0;
     if (check_structure(d) != GF_OK) return 0;
+    const gf_desc db = batch_desc(d);
+    d = &db;
     for (int i = 0; i < b->count; ++i)
         if (check_stamp(d, b->H[i], b->W[i]) != GF_OK) return 0;
     Structure S;
@@ -1498,6 +1545,8 @@ static gf_status eval_batch_impl(const gf_desc* d, const gf_batch* b, const doub
 {
     gf_status r = check_structure(d);
     if (r != GF_OK) return r;
+    const gf_desc db = batch_desc(d);
+    d = &db;
     if (!b || b->count < 1 || !b->H || !b->W) return fail(GF_EINVAL, "bad batch");
     for (int i = 0; i < b->count; ++i)
         if ((r = check_stamp(d, b->H[i], b->W[i])) != GF_OK) return r;
@@ -1599,10 +1648,12 @@ static gf_status lm_fit_impl(const gf_desc* d, const gf_batch* b, double* params
                              const uint8_t* fixed, const double* lo, const double* hi,
                              const float* img, const float* sig, const float* psf,
                              const gf_lm_opts* opts, gf_lm_result* res, void* ws, size_t ws_bytes,
-                             gf_stream stream)
+                             gf_stream stream, bool batched)
 {
     gf_status r = check_structure(d);
     if (r != GF_OK) return r;
+    const gf_desc db = batched ? batch_desc(d) : *d;
+    d = &db;
     if (!b || b->count < 1 || !b->H || !b->W) return fail(GF_EINVAL, "bad batch");
     for (int i = 0; i < b->count; ++i)
         if ((r = check_stamp(d, b->H[i], b->W[i])) != GF_OK) return r;
@@ -1640,7 +1691,7 @@ static gf_status lm_fit_impl(const gf_desc* d, const gf_batch* b, double* params
     set_grids(at_, L, L.rungs);
     // the direct path and the one-CTA FFT reduce the trial chi^2 inside the
     // convolution (no convolved trial model written)
-    at_.conv_chi2 = (pl.method == GF_CONV_DIRECT || (pl.method == GF_CONV_FFT && pl.small)) ? 1 : 0;
+    at_.conv_chi2 = (pl.method == GF_CONV_DIRECT || pl.small) ? 1 : 0;
     if (at_.conv_chi2) at_.max_trial_slots = (int)std::min<long long>(L.max_wb, INT32_MAX);
     // each pass walks the list of stamps in its phase, rebuilt every body
     aj.wl.n = at<int>(ws, L.wl_n[0]);
@@ -1896,7 +1947,7 @@ gf_status gf_lm_fit_batch(const gf_desc* d, const gf_batch* b, double* params,
                           size_t ws_bytes, gf_stream stream)
 {
     return lm_fit_impl(d, b, params, fixed, nullptr, nullptr, img, sig, psf, opts, res, ws,
-                       ws_bytes, stream);
+                       ws_bytes, stream, true);
 }
 
 // The batch of a multi-start fit: stamp i repeated `starts` times (entry
@@ -1962,7 +2013,7 @@ gf_status gf_lm_fit_multistart(const gf_desc* d, const gf_batch* b, int starts,
     std::vector<double> p(starts_host, starts_host + (size_t)n * ns);
     std::vector<gf_lm_result> res((size_t)n);
     if ((r = lm_fit_impl(d, &m.b, p.data(), fixed, nullptr, nullptr, img, sig, psf, opts, res.data(),
-                         ws, ws_bytes, stream)) != GF_OK)
+                         ws, ws_bytes, stream, true)) != GF_OK)
         return r;
     // per stamp the fit with the lowest finite chi^2, the earliest start on ties
     for (int i = 0; i < b->count; ++i) {
@@ -1997,7 +2048,7 @@ gf_status gf_lm_fit(const gf_desc* d, double* params, const uint8_t* fixed, cons
     b.pix_off = &zero;
     b.psf_off = &zero;
     return lm_fit_impl(d, &b, params, fixed, lo, hi, img, sig, psf, opts, res, ws, ws_bytes,
-                       stream);
+                       stream, false);
 }
 
 }  // extern "C"
