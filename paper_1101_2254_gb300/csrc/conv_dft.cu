@@ -56,27 +56,44 @@ __device__ __forceinline__ float2 cmulf(float2 a, float2 b)
     return make_float2(a.x * b.x - a.y * b.y, a.x * b.y + a.y * b.x);
 }
 
-// e >= 0 and below 64 * 4096 for every stage, so 32-bit arithmetic suffices
-__device__ __forceinline__ float2 twiddle(const DftStage& s, int e)
+// Eight consecutive values r8 .. r8 + 7 of a row, zeros past R.  `in` points at
+// the row's value 0 and steps by `step` values (so an element costs an addition,
+// not the division and the 64-bit products of its whole index).
+//   MODE 0 complex values, 1 a real grid (`lim` of its columns left: value r is
+//   inside while r step < lim), 2 complex values times the PSF spectrum.
+template <int MODE>
+__device__ __forceinline__ void load8(float2 (&v)[8], const float2* in, const float2* h, int step, int r8, int R,
+                                      int lim)
 {
-    e %= s.tw_N;
-    float2 w = s.tw[e];
-    if (s.tw_sign > 0.0f) w.y = -w.y;
-    return w;
+    if (MODE == 1) {
+        const float* re = reinterpret_cast<const float*>(in);
+#pragma unroll
+        for (int j = 0; j < 8; ++j) {
+            const int o = (r8 + j) * step;
+            v[j] = make_float2(r8 + j < R && o < lim ? re[o] : 0.0f, 0.0f);
+        }
+        return;
+    }
+#pragma unroll
+    for (int j = 0; j < 8; ++j) v[j] = r8 + j < R ? in[(r8 + j) * step] : make_float2(0.0f, 0.0f);
+    if (MODE == 2) {
+        float2 w[8];
+#pragma unroll
+        for (int j = 0; j < 8; ++j) w[j] = r8 + j < R ? h[(r8 + j) * step] : make_float2(0.0f, 0.0f);
+#pragma unroll
+        for (int j = 0; j < 8; ++j) v[j] = cmulf(v[j], w[j]);
+    }
 }
 
-__device__ __forceinline__ float2 in_a(const DftStage& s, int p, int l, int r, int q)
+// the same of a contiguous row with an even R: two values a load
+__device__ __forceinline__ void load8_pairs(float2 (&v)[8], const float2* in, int r8, int R)
 {
-    if (s.in_mode == 1) {
-        const int y = l, x = r * s.in_xdigit + q;
-        if (y >= s.in_rows || x >= s.in_cols) return make_float2(0.f, 0.f);
-        return make_float2(s.in_real[(long long)p * s.in_real_pstride + (long long)y * s.in_ld + x],
-                           0.f);
+#pragma unroll
+    for (int j = 0; j < 8; j += 2) {
+        const float4 t = r8 + j < R ? *reinterpret_cast<const float4*>(in + r8 + j) : make_float4(0.f, 0.f, 0.f, 0.f);
+        v[j] = make_float2(t.x, t.y);
+        v[j + 1] = make_float2(t.z, t.w);
     }
-    const long long idx = ((long long)l * s.R + r) * s.Q + q;
-    float2 v = s.in[(long long)p * s.in_pstride + idx];
-    if (s.in_mode == 2) v = cmulf(v, s.hhat[(long long)(p / s.nchan) * s.in_pstride + idx]);
-    return v;
 }
 
 // One contraction stage on the tensor cores (see the top of the file).
@@ -137,30 +154,50 @@ __global__ void __launch_bounds__(NT) k_dft_tc(DftStage s, int tpc, unsigned lon
             const int row = tid & (TM - 1), half = tid >> 7;
             const long long g = g0 + row;
             const int rbeg = half * (Kp / 2), rend = rbeg + Kp / 2;
-            int l = 0, q = 0;
-            if (ORIENT_A && g < rows) {
-                l = (int)(g / s.Q);
-                q = (int)(g - (long long)l * s.Q);
+            // the row's value 0, the step between its values and (real grid) the
+            // columns left; a row outside counts no value
+            const float2* in = s.in;
+            const float2* h = s.hhat;
+            int step = 1, lim = 0, Rv = g < rows ? R : 0;
+            if (ORIENT_A) {
+                const unsigned l = (unsigned)g / (unsigned)s.Q, q = (unsigned)g - l * (unsigned)s.Q;
+                if (s.in_mode == 1) {
+                    in = reinterpret_cast<const float2*>(s.in_real + (long long)p * s.in_real_pstride +
+                                                         (long long)l * s.in_ld + q);
+                    step = s.in_xdigit;
+                    lim = s.in_cols - (int)q;
+                    if ((int)l >= s.in_rows) Rv = 0;
+                } else {
+                    const long long at = (long long)l * R * s.Q + q;
+                    in += (long long)p * s.in_pstride + at;
+                    if (s.in_mode == 2) h += (long long)(p / s.nchan) * s.in_pstride + at;
+                    step = s.Q;
+                }
+            } else {
+                in += (long long)p * s.in_pstride + g * R;
             }
+            const bool pairs = !ORIENT_A && (R & 1) == 0 && (reinterpret_cast<uintptr_t>(s.in) & 15) == 0 &&
+                               (s.in_pstride & 1) == 0;
             for (int r8 = rbeg; r8 < rend; r8 += 8) {
-                __align__(16) __nv_bfloat16 h[4][8];
+                float2 v[8];
+                if (!ORIENT_A && pairs)
+                    load8_pairs(v, in, r8, Rv);
+                else if (!ORIENT_A || s.in_mode == 0)
+                    load8<0>(v, in, h, step, r8, Rv, lim);
+                else if (s.in_mode == 1)
+                    load8<1>(v, in, h, step, r8, Rv, lim);
+                else
+                    load8<2>(v, in, h, step, r8, Rv, lim);
+                __align__(16) __nv_bfloat16 pl4[4][8];
 #pragma unroll
                 for (int j = 0; j < 8; ++j) {
-                    const int r = r8 + j;
-                    float2 v = make_float2(0.f, 0.f);
-                    if (g < rows && r < R) {
-                        if (ORIENT_A)
-                            v = in_a(s, p, l, r, q);
-                        else
-                            v = s.in[(long long)p * s.in_pstride + g * R + r];
-                    }
-                    split_bf16(v.x, h[0][j], h[1][j]);
-                    split_bf16(v.y, h[2][j], h[3][j]);
+                    split_bf16(v[j].x, pl4[0][j], pl4[1][j]);
+                    split_bf16(v[j].y, pl4[2][j], pl4[3][j]);
                 }
                 const int o = cofs(row, r8, Kp);
 #pragma unroll
                 for (int pl = 0; pl < 4; ++pl)
-                    *reinterpret_cast<uint4*>(Ap + pl * TM * Kp + o) = *reinterpret_cast<const uint4*>(h[pl]);
+                    *reinterpret_cast<uint4*>(Ap + pl * TM * Kp + o) = *reinterpret_cast<const uint4*>(pl4[pl]);
             }
         }
         asm volatile("fence.proxy.async.shared::cta;");
@@ -229,36 +266,78 @@ __global__ void __launch_bounds__(NT) k_dft_tc(DftStage s, int tpc, unsigned lon
             const long long g = g0 + row;
             int l = 0, q = 0;
             if (ORIENT_A) {
-                l = (int)(g / s.Q);
-                q = (int)(g - (long long)l * s.Q);
+                l = (int)((unsigned)g / (unsigned)s.Q);
+                q = (int)((unsigned)g - (unsigned)l * (unsigned)s.Q);
             }
+            // the twiddle of output k is w_N^{k m}, one m for the row: its exponent
+            // steps by m mod N
+            const int k00 = khalf * (Rp / 2);
+            int m = 0, ex = 0;
+            if (s.tw_mode) {
+                m = s.tw_mode == 1 ? (q / s.tw_div) % s.tw_mod : s.tw_mode == 2 ? l : (int)((unsigned)g % (unsigned)s.tw_mod);
+                m %= s.tw_N;
+                ex = (k00 * m) % s.tw_N;
+            }
+            const float2* tw = s.tw;
+            const float tws = s.tw_sign > 0.0f ? -1.0f : 1.0f;
+            // the row's output 0 (real crop: column q of output row l, outside it
+            // where the row is)
+            float2* out = nullptr;
+            float* outr = nullptr;
+            int x = 0;
+            bool live = g < rows;
+            if (ORIENT_A && s.out_mode == 1) {
+                const int y = l - s.crop_y0;
+                live = live && y >= 0 && y < s.crop_H;
+                outr = s.out_real + (long long)p * s.out_real_pstride + (long long)y * s.crop_W;
+                x = k00 * s.out_xdigit + q - s.crop_x0;
+            } else {
+                out = s.out + (long long)p * s.out_pstride +
+                      (ORIENT_A ? ((long long)l * R + k00) * s.Q + q : g * R + k00);
+            }
+            const bool pairs = !ORIENT_A && (R & 1) == 0 && (reinterpret_cast<uintptr_t>(s.out) & 15) == 0 &&
+                               (s.out_pstride & 1) == 0;
             const uint32_t taddr = tmem + ((uint32_t)(quarter * 32) << 16);
-            for (int k0 = khalf * (Rp / 2); k0 < (khalf + 1) * (Rp / 2); k0 += 8) {
+            for (int k0 = k00; k0 < k00 + Rp / 2; k0 += 8) {
                 float re[8], im[8];
                 tmem_ld8(taddr + k0, re);
                 tmem_ld8(taddr + Rp + k0, im);
-                if (g >= rows) continue;
+                float2 v[8];
+                if (s.tw_mode) {
+                    float2 w[8];
 #pragma unroll
-                for (int j = 0; j < 8; ++j) {
-                    const int k = k0 + j;
-                    if (k >= R) continue;
-                    float2 v = make_float2(re[j], im[j]);
-                    if (ORIENT_A) {
-                        if (s.tw_mode == 1)
-                            v = cmulf(v, twiddle(s, k * ((q / s.tw_div) % s.tw_mod)));
-                        else if (s.tw_mode == 2)
-                            v = cmulf(v, twiddle(s, l * k));
-                        if (s.out_mode == 0) {
-                            s.out[(long long)p * s.out_pstride + ((long long)l * R + k) * s.Q + q] = v;
-                        } else {
-                            const int y = l - s.crop_y0, x = k * s.out_xdigit + q - s.crop_x0;
-                            if (y >= 0 && y < s.crop_H && x >= 0 && x < s.crop_W)
-                                s.out_real[(long long)p * s.out_real_pstride + (long long)y * s.crop_W + x] = v.x;
-                        }
-                    } else {
-                        if (s.tw_mode == 3) v = cmulf(v, twiddle(s, (int)(g % s.tw_mod) * k));
-                        s.out[(long long)p * s.out_pstride + g * R + k] = v;
+                    for (int j = 0; j < 8; ++j) {
+                        w[j] = tw[ex];
+                        ex += m;
+                        if (ex >= s.tw_N) ex -= s.tw_N;
                     }
+#pragma unroll
+                    for (int j = 0; j < 8; ++j) v[j] = cmulf(make_float2(re[j], im[j]), make_float2(w[j].x, tws * w[j].y));
+                } else {
+#pragma unroll
+                    for (int j = 0; j < 8; ++j) v[j] = make_float2(re[j], im[j]);
+                }
+                if (!live) continue;
+                if (ORIENT_A && s.out_mode == 1) {
+#pragma unroll
+                    for (int j = 0; j < 8; ++j) {
+                        if (k0 + j < R && x >= 0 && x < s.crop_W) outr[x] = v[j].x;
+                        x += s.out_xdigit;
+                    }
+                } else if (ORIENT_A) {
+#pragma unroll
+                    for (int j = 0; j < 8; ++j)
+                        if (k0 + j < R) out[(k0 - k00 + j) * s.Q] = v[j];
+                } else if (pairs) {
+#pragma unroll
+                    for (int j = 0; j < 8; j += 2)
+                        if (k0 + j < R)
+                            *reinterpret_cast<float4*>(out + (k0 - k00) + j) =
+                                make_float4(v[j].x, v[j].y, v[j + 1].x, v[j + 1].y);
+                } else {
+#pragma unroll
+                    for (int j = 0; j < 8; ++j)
+                        if (k0 + j < R) out[(k0 - k00) + j] = v[j];
                 }
             }
         }
