@@ -62,24 +62,41 @@ __device__ __forceinline__ void unpack8(const uint4 u, float* f)
 inline int blocks(long long n, int t) { return (int)((n + t - 1) / t); }
 
 // ---------------------------------------------------------------- forward
-// fc1: thread = (b, o); input the flattened conv4 output (bf16), output float32 after ReLU
+// fc1: thread = (NB samples, o); input the flattened conv4 output (bf16), output
+// float32 after ReLU.  A lane's weights are a row of their own (32 sectors a load),
+// which is what bounds it, so NB samples share them; four loads stay in flight.
+// 8,192 stamps (NB 4): 257 us -> 101.  Below 2,048 samples a sample a thread: four would
+// leave most SMs without a block.
+template <int NB>
 __global__ void k_fc1_fwd(const __nv_bfloat16* __restrict__ a3, const __nv_bfloat16* __restrict__ w,
                           const float* __restrict__ master, float* __restrict__ h, int B)
 {
     const int item = blockIdx.x * blockDim.x + threadIdx.x;
-    if (item >= B * 32) return;
-    const int b = item / 32, o = item - b * 32;
-    const __nv_bfloat16* xr = a3 + (long long)b * 2048;
+    const int b0 = (item >> 5) * NB, o = item & 31;
+    if (b0 >= B) return;
+    const __nv_bfloat16* xr[NB];
+    float acc[NB];
+#pragma unroll
+    for (int q = 0; q < NB; ++q) {
+        xr[q] = a3 + (long long)min(b0 + q, B - 1) * 2048;
+        acc[q] = master[FC1_B + o];
+    }
     const __nv_bfloat16* wr = w + FC1_W + o * 2048;
-    float acc = master[FC1_B + o];
+#pragma unroll 4
     for (int i = 0; i < 2048; i += 8) {
-        float xv[8], wv[8];
-        unpack8(*reinterpret_cast<const uint4*>(xr + i), xv);
+        float wv[8];
         unpack8(*reinterpret_cast<const uint4*>(wr + i), wv);
 #pragma unroll
-        for (int j = 0; j < 8; ++j) acc = fmaf(xv[j], wv[j], acc);
+        for (int q = 0; q < NB; ++q) {
+            float xv[8];
+            unpack8(*reinterpret_cast<const uint4*>(xr[q] + i), xv);
+#pragma unroll
+            for (int j = 0; j < 8; ++j) acc[q] = fmaf(xv[j], wv[j], acc[q]);
+        }
     }
-    h[item] = fmaxf(acc, 0.0f);
+#pragma unroll
+    for (int q = 0; q < NB; ++q)
+        if (b0 + q < B) h[(b0 + q) * 32 + o] = fmaxf(acc[q], 0.0f);
 }
 
 // fc2: thread = (b, j); linear output
@@ -127,11 +144,13 @@ __global__ void k_fc2_bwd_w(const float* __restrict__ gy, const float* __restric
     if (item < NOUT * 32) {
         const int j = item / 32, o = item - j * 32;
         float s = 0.0f;
+#pragma unroll 16  // (the loads of 16 samples in flight; the sum stays in order)
         for (int b = 0; b < B; ++b) s = fmaf(gy[b * NOUT + j], h[b * 32 + o], s);
         grad[FC2_W + item] = s;
     } else if (item < NOUT * 32 + NOUT) {
         const int j = item - NOUT * 32;
         float s = 0.0f;
+#pragma unroll 16
         for (int b = 0; b < B; ++b) s += gy[b * NOUT + j];
         grad[FC2_B + j] = s;
     }
@@ -157,11 +176,13 @@ __global__ void k_fc1_bwd_w(const float* __restrict__ gh, const __nv_bfloat16* _
     if (item < 32 * 2048) {
         const int o = item / 2048, i = item - o * 2048;
         float s = 0.0f;
+#pragma unroll 16
         for (int b = 0; b < B; ++b) s = fmaf(gh[b * 32 + o], __bfloat162float(a3[(long long)b * 2048 + i]), s);
         grad[FC1_W + item] = s;
     } else if (item < 32 * 2048 + 32) {
         const int o = item - 32 * 2048;
         float s = 0.0f;
+#pragma unroll 16
         for (int b = 0; b < B; ++b) s += gh[b * 32 + o];
         grad[FC1_B + o] = s;
     }
@@ -184,57 +205,69 @@ __global__ void k_fc1_bwd_x(const float* __restrict__ gh, const __nv_bfloat16* _
 
 // Weight gradients of the first convolution (one input channel, nine taps per
 // output channel: too narrow for the tensor cores), first stage: block =
-// (output channel co, input channel ci, chunk of the batch); threads stride over
-// (b, oy, ox) keeping the nine tap sums (and the bias sum); a fixed tree merges
-// the threads.  gout is channels-last (b, oy, ox, co).
+// (8 output channels, chunk of the batch); threads stride over (b, oy, ox),
+// keeping for each channel the nine tap sums and the bias sum; a fixed tree merges
+// the threads.  gout is channels-last (b, oy, ox, co), so 8 channels are the 32
+// bytes that a pixel's read fetches in any case, and the nine inputs are read once
+// for the 8 (a block per channel: 174 us on 512 stamps, 74 now).
 constexpr int WG_THREADS = 256;
+constexpr int WG_CO = 8;  // channels a block
 
 __global__ void __launch_bounds__(WG_THREADS) k_conv_bwd_w(const float* __restrict__ gout,
                                                             const __nv_bfloat16* __restrict__ xin,
-                                                            float* __restrict__ part, int B,
-                                                            int cin, int hin, int cout, int hout,
-                                                            int nchunk)
+                                                            float* __restrict__ part, int B, int hin,
+                                                            int cout, int hout, int nchunk)
 {
     __shared__ float red[10][WG_THREADS];
-    const int co = blockIdx.x / cin, ci = blockIdx.x - co * cin, chunk = blockIdx.y;
-    const int npix = hout * hout;
+    const int co0 = blockIdx.x * WG_CO, chunk = blockIdx.y;
+    const int npix = hout * hout, lho = __ffs(hout) - 1;  // (a power of two)
     const long long total = (long long)B * npix;
     const long long per = (total + nchunk - 1) / nchunk;
     const long long i0 = chunk * per, i1 = min(total, i0 + per);
-    float s[10];
+    float s[WG_CO][10];
 #pragma unroll
-    for (int k = 0; k < 10; ++k) s[k] = 0.0f;
+    for (int j = 0; j < WG_CO; ++j)
+#pragma unroll
+        for (int k = 0; k < 10; ++k) s[j][k] = 0.0f;
     for (long long it = i0 + threadIdx.x; it < i1; it += WG_THREADS) {
-        const int b = (int)(it / npix), pix = (int)(it - (long long)b * npix);
-        const int oy = pix / hout, ox = pix - oy * hout;
-        const float g = gout[((long long)b * npix + pix) * cout + co];
-        if (g == 0.0f) continue;
-        s[9] += g;
-        const __nv_bfloat16* xb = xin + ((long long)b * cin + ci) * hin * hin;
+        const int b = (int)(it >> (2 * lho)), pix = (int)it & (npix - 1);
+        const int oy = pix >> lho, ox = pix & (hout - 1);
+        const float4* gp = reinterpret_cast<const float4*>(gout + it * cout + co0);
+        const float4 g0 = gp[0], g1 = gp[1];
+        const float g[WG_CO] = {g0.x, g0.y, g0.z, g0.w, g1.x, g1.y, g1.z, g1.w};
+        const __nv_bfloat16* xb = xin + (long long)b * hin * hin;
+        float x[9];
+        bool in[9];  // taps inside the image
 #pragma unroll
-        for (int ky = 0; ky < 3; ++ky) {
-            const int iy = 2 * oy - 1 + ky;
-            if (iy < 0 || iy >= hin) continue;
+        for (int t = 0; t < 9; ++t) {
+            const int iy = 2 * oy - 1 + t / 3, ix = 2 * ox - 1 + t % 3;
+            in[t] = iy >= 0 && iy < hin && ix >= 0 && ix < hin;
+            x[t] = in[t] ? __bfloat162float(xb[iy * hin + ix]) : 0.0f;
+        }
 #pragma unroll
-            for (int kx = 0; kx < 3; ++kx) {
-                const int ix = 2 * ox - 1 + kx;
-                if (ix < 0 || ix >= hin) continue;
-                s[ky * 3 + kx] = fmaf(g, __bfloat162float(xb[iy * hin + ix]), s[ky * 3 + kx]);
-            }
+        for (int j = 0; j < WG_CO; ++j) {
+            if (g[j] == 0.0f) continue;  // (also where the input is not finite)
+            s[j][9] += g[j];
+#pragma unroll
+            for (int t = 0; t < 9; ++t)
+                if (in[t]) s[j][t] = fmaf(g[j], x[t], s[j][t]);
         }
     }
 #pragma unroll
-    for (int k = 0; k < 10; ++k) red[k][threadIdx.x] = s[k];
-    __syncthreads();
-    for (int w = WG_THREADS / 2; w > 0; w >>= 1) {
-        if (threadIdx.x < w)
+    for (int j = 0; j < WG_CO; ++j) {
+        __syncthreads();  // (the sums of the channel before are out)
 #pragma unroll
-            for (int k = 0; k < 10; ++k) red[k][threadIdx.x] += red[k][threadIdx.x + w];
+        for (int k = 0; k < 10; ++k) red[k][threadIdx.x] = s[j][k];
         __syncthreads();
+        for (int w = WG_THREADS / 2; w > 0; w >>= 1) {
+            if (threadIdx.x < w)
+#pragma unroll
+                for (int k = 0; k < 10; ++k) red[k][threadIdx.x] += red[k][threadIdx.x + w];
+            __syncthreads();
+        }
+        // part layout: [chunk][co][10]
+        if (threadIdx.x < 10) part[((long long)chunk * cout + co0 + j) * 10 + threadIdx.x] = red[threadIdx.x][0];
     }
-    // part layout: [chunk][co][ci][10]
-    if (threadIdx.x < 10)
-        part[(((long long)chunk * cout + co) * cin + ci) * 10 + threadIdx.x] = red[threadIdx.x][0];
 }
 
 // second stage: the chunks summed in order into the packed master layout
@@ -1087,7 +1120,10 @@ cudaError_t cnn_prepare(const float* w, const float* x, int B, const CnnBuffers&
 
 cudaError_t cnn_forward_fc(const float* w, int B, const CnnBuffers& cb, float* y, cudaStream_t s)
 {
-    k_fc1_fwd<<<blocks((long long)B * 32, 256), 256, 0, s>>>(cb.a3, cb.wp, w, cb.h, B);
+    if (B >= 2048)  // (fewer samples leave SMs idle at four a thread)
+        k_fc1_fwd<4><<<blocks((long long)(B + 3) / 4 * 32, 256), 256, 0, s>>>(cb.a3, cb.wp, w, cb.h, B);
+    else
+        k_fc1_fwd<1><<<blocks((long long)B * 32, 128), 128, 0, s>>>(cb.a3, cb.wp, w, cb.h, B);
     GF_COUNT_LAUNCH();
     k_fc2_fwd<<<blocks((long long)B * NOUT, 256), 256, 0, s>>>(cb.h, cb.wp, w, y ? y : cb.y, B);
     GF_COUNT_LAUNCH();
@@ -1116,8 +1152,9 @@ cudaError_t cnn_backward(const float* t, int B, float* loss, float* grad, const 
     const ConvL L = CONV[0];
     const long long total = (long long)B * L.hout * L.hout;
     const int nchunk = (int)std::min<long long>(std::max<long long>(1, 2048 / (L.cout * L.cin)), total);
-    k_conv_bwd_w<<<dim3(L.cout * L.cin, nchunk), WG_THREADS, 0, s>>>(cb.g0, cb.x, cb.part, B, L.cin, L.hin,
-                                                                     L.cout, L.hout, nchunk);
+    static_assert(CONV[0].cin == 1 && CONV[0].cout % WG_CO == 0, "one input channel, whole blocks of outputs");
+    k_conv_bwd_w<<<dim3(L.cout / WG_CO, nchunk), WG_THREADS, 0, s>>>(cb.g0, cb.x, cb.part, B, L.hin, L.cout,
+                                                                     L.hout, nchunk);
     GF_COUNT_LAUNCH();
     k_conv_bwd_w_sum<<<blocks((long long)L.cout * L.cin * 10, 256), 256, 0, s>>>(cb.part, grad, L.cin, L.cout,
                                                                                 nchunk, L.woff, L.boff);

@@ -28,7 +28,8 @@
 // accumulator holds its 128 x cout partial sums); the chunks' partials are
 // added in chunk order by a second kernel, so the result does not depend on
 // scheduling.  Input gradient: a persistent CTA walks tiles of 128 input
-// pixels, with the weights (cin x 9 cout) resident in shared memory.
+// pixels of one parity class, with the weights (cin x 9 cout) resident in shared
+// memory.
 #include <math.h>
 #include <stdint.h>
 
@@ -97,9 +98,13 @@ struct ConvBwd {
 };
 
 // ------------------------------------------------------------ weight gradient
-// grid (n-tiles, chunks); NCO = cout
+// grid (n-tiles, chunks); NCO = cout.  A block's values are loaded into registers
+// while the MMAs of the one before run, and rows are split by shifts (a 64-bit
+// division a row of each piece before).  512 stamps, layer 4
+// 48 us -> 45, layers 3 and 2 together 423 -> 221 (of which the channels of a
+// staged row shared by four threads 360 -> 221).
 template <int NCO>
-__global__ void __launch_bounds__(BT_THREADS) k_conv_dw_tc(ConvBwd a)
+__global__ void __launch_bounds__(BT_THREADS, 2) k_conv_dw_tc(ConvBwd a)
 {
     extern __shared__ __align__(128) unsigned char smem_raw[];
     __shared__ __align__(8) uint64_t bar;
@@ -116,83 +121,90 @@ __global__ void __launch_bounds__(BT_THREADS) k_conv_dw_tc(ConvBwd a)
     const uint32_t idesc = idesc_bf16(128, NCO);
     const uint32_t xa = smem_addr(Xs), ga = smem_addr(Gs);
     constexpr uint32_t PLANE = NCO * BT_KB * 2;  // bytes per G plane
-    const int hw = a.hout * a.hout, n0 = blockIdx.x * 128, nw = 9 * a.cin;
-    const long long M = (long long)a.B * hw;
+    // (the layers' sides and channels are powers of two: rows split by shifts)
+    const int lho = __ffs(a.hout) - 1, lci = __ffs(a.cin) - 1;
+    const int n0 = blockIdx.x * 128, nw = 9 * a.cin;
+    const long long M = (long long)a.B << (2 * lho);
     const long long nkb = (M + BT_KB - 1) / BT_KB;
     const long long kb0 = nkb * blockIdx.y / a.nchunk, kb1 = nkb * (blockIdx.y + 1) / a.nchunk;
-    uint32_t parity = 0;
-    bool failed = false;
-    for (long long kb = kb0; kb < kb1 && !failed; ++kb) {
-        const long long mb = kb * BT_KB;
-        // A: rows n of this tile x 64 m (an 8 x 8 block per item, transposed)
-        for (int it = tid; it < 16 * 8 + (NCO / 8) * 8; it += BT_THREADS) {
-            if (it < 128) {
-                const int ng = it >> 3, mg = it & 7;
-                const int n = n0 + 8 * ng;
-                __nv_bfloat16 v[8][8];  // [m][n]
-                if (n < nw) {
-                    const int tap = n / a.cin, ci = n - tap * a.cin;
-                    const int ky = tap / 3, kx = tap - 3 * ky;
+    // this thread's item of a block: an 8 x 8 piece of A (rows n x m; threads 0-127) or
+    // a CB x 8 piece of B (channels x m; the others)
+    constexpr int CB = NCO / 16;  // channels of a B item
+    static_assert(BT_THREADS == 256 && (CB == 4 || CB == 8), "an item a thread");
+    const int ng = tid >> 3, mg = tid & 7, cg = (tid - 128) >> 3;
+    const bool is_a = tid < 128;
+    const int n = n0 + 8 * ng, tap = n >> lci, ci = n & (a.cin - 1);
+    const int ky = tap / 3, kx = tap - 3 * ky;
+    uint4 ld[2 * CB];  // A: 8 bf16 a row m in ld[0..7]; B: CB floats a row m
+    auto load = [&](long long kb) {
+        const long long m0 = kb * BT_KB + 8 * mg;
 #pragma unroll
-                    for (int i = 0; i < 8; ++i) {
-                        const long long m = mb + 8 * mg + i;
-                        uint4 u = make_uint4(0u, 0u, 0u, 0u);
-                        if (m < M) {
-                            const int b = (int)(m / hw), pix = (int)(m - (long long)b * hw);
-                            const int oy = pix / a.hout, ox = pix - oy * a.hout;
-                            const int iy = 2 * oy - 1 + ky, ix = 2 * ox - 1 + kx;
-                            if (iy >= 0 && iy < a.hin && ix >= 0 && ix < a.hin)
-                                u = *reinterpret_cast<const uint4*>(
-                                    a.x + (((long long)b * a.hin + iy) * a.hin + ix) * a.cin + ci);
-                        }
-                        const __nv_bfloat16* h = reinterpret_cast<const __nv_bfloat16*>(&u);
-#pragma unroll
-                        for (int j = 0; j < 8; ++j) v[i][j] = h[j];
-                    }
-                } else {
-                    // the bias row (ones where m is in range) and the padding rows
-#pragma unroll
-                    for (int i = 0; i < 8; ++i) {
-                        const bool in = mb + 8 * mg + i < M;
-#pragma unroll
-                        for (int j = 0; j < 8; ++j)
-                            v[i][j] = __float2bfloat16_rn((n + j == nw && in) ? 1.0f : 0.0f);
-                    }
-                }
-#pragma unroll
-                for (int j = 0; j < 8; ++j) {
-                    __nv_bfloat16 r[8];
-#pragma unroll
-                    for (int i = 0; i < 8; ++i) r[i] = v[i][j];
-                    *reinterpret_cast<uint4*>(Xs + cofs(8 * ng + j, 8 * mg, BT_KB)) = pack8(r);
+        for (int i = 0; i < 8; ++i) {
+            const long long m = m0 + i;
+            const uint4 z = make_uint4(0u, 0u, 0u, 0u);
+            if (is_a) {
+                ld[i] = z;
+                if (n < nw && m < M) {
+                    const int bs = (int)(m >> (2 * lho)), pix = (int)m & ((1 << (2 * lho)) - 1);
+                    const int oy = pix >> lho, ox = pix & (a.hout - 1);
+                    const int iy = 2 * oy - 1 + ky, ix = 2 * ox - 1 + kx;
+                    if (iy >= 0 && iy < a.hin && ix >= 0 && ix < a.hin)
+                        ld[i] = *reinterpret_cast<const uint4*>(
+                            a.x + (((long long)bs * a.hin + iy) * a.hin + ix) * a.cin + ci);
                 }
             } else {
-                // B: G rows m x 8 channels, split into three planes and transposed
-                const int q = it - 128, cg = q >> 3, mg = q & 7;
-                __nv_bfloat16 hi[8][8], mid[8][8], lo[8][8];  // [co][m]
+                const uint4* src = reinterpret_cast<const uint4*>(a.g + m * NCO + CB * cg);
+#pragma unroll
+                for (int h = 0; h < CB / 4; ++h) ld[i * (CB / 4) + h] = m < M ? src[h] : z;
+            }
+        }
+    };
+    uint32_t parity = 0;
+    bool failed = false;
+    if (kb0 < kb1) load(kb0);
+    for (long long kb = kb0; kb < kb1 && !failed; ++kb) {
+        const long long mb = kb * BT_KB;
+        if (is_a) {
+            __nv_bfloat16 v[8][8];  // [m][n]
+            if (n < nw) {
 #pragma unroll
                 for (int i = 0; i < 8; ++i) {
-                    const long long m = mb + 8 * mg + i;
-                    float f[8];
-                    if (m < M) {
-                        const float4* src = reinterpret_cast<const float4*>(a.g + m * NCO + 8 * cg);
-                        const float4 p0 = src[0], p1 = src[1];
-                        f[0] = p0.x; f[1] = p0.y; f[2] = p0.z; f[3] = p0.w;
-                        f[4] = p1.x; f[5] = p1.y; f[6] = p1.z; f[7] = p1.w;
-                    } else {
+                    const __nv_bfloat16* h = reinterpret_cast<const __nv_bfloat16*>(&ld[i]);
 #pragma unroll
-                        for (int j = 0; j < 8; ++j) f[j] = 0.0f;
-                    }
-#pragma unroll
-                    for (int j = 0; j < 8; ++j) split3(f[j], hi[j][i], mid[j][i], lo[j][i]);
+                    for (int j = 0; j < 8; ++j) v[i][j] = h[j];
                 }
+            } else {
+                // the bias row (ones where m is in range) and the padding rows
 #pragma unroll
-                for (int j = 0; j < 8; ++j) {
-                    const int o = cofs(8 * cg + j, 8 * mg, BT_KB);
-                    *reinterpret_cast<uint4*>(Gs + o) = pack8(hi[j]);
-                    *reinterpret_cast<uint4*>(Gs + PLANE / 2 + o) = pack8(mid[j]);
-                    *reinterpret_cast<uint4*>(Gs + PLANE + o) = pack8(lo[j]);
+                for (int i = 0; i < 8; ++i) {
+                    const bool in = mb + 8 * mg + i < M;
+#pragma unroll
+                    for (int j = 0; j < 8; ++j)
+                        v[i][j] = __float2bfloat16_rn((n + j == nw && in) ? 1.0f : 0.0f);
                 }
+            }
+#pragma unroll
+            for (int j = 0; j < 8; ++j) {
+                __nv_bfloat16 r[8];
+#pragma unroll
+                for (int i = 0; i < 8; ++i) r[i] = v[i][j];
+                *reinterpret_cast<uint4*>(Xs + cofs(8 * ng + j, 8 * mg, BT_KB)) = pack8(r);
+            }
+        } else {
+            // G rows m x CB channels, split into three planes and transposed
+            __nv_bfloat16 hi[CB][8], mid[CB][8], lo[CB][8];  // [co][m]
+#pragma unroll
+            for (int i = 0; i < 8; ++i) {
+                const float* f = reinterpret_cast<const float*>(&ld[i * (CB / 4)]);
+#pragma unroll
+                for (int j = 0; j < CB; ++j) split3(f[j], hi[j][i], mid[j][i], lo[j][i]);
+            }
+#pragma unroll
+            for (int j = 0; j < CB; ++j) {
+                const int o = cofs(CB * cg + j, 8 * mg, BT_KB);
+                *reinterpret_cast<uint4*>(Gs + o) = pack8(hi[j]);
+                *reinterpret_cast<uint4*>(Gs + PLANE / 2 + o) = pack8(mid[j]);
+                *reinterpret_cast<uint4*>(Gs + PLANE + o) = pack8(lo[j]);
             }
         }
         mma_fence_sync();
@@ -204,6 +216,7 @@ __global__ void __launch_bounds__(BT_THREADS) k_conv_dw_tc(ConvBwd a)
                          (kb > kb0 || ks > 0 || p > 0) ? 1 : 0);
             mma_commit(bar_a);
         }
+        if (kb + 1 < kb1) load(kb + 1);  // in flight while the MMAs run
         const bool done = mbar_wait(bar_a, parity);
         parity ^= 1u;
         asm volatile("tcgen05.fence::after_thread_sync;");
@@ -253,7 +266,8 @@ __global__ void k_conv_dw_sum(const float* __restrict__ part, float* __restrict_
 }
 
 // ------------------------------------------------------------- input gradient
-// persistent grid over tiles of 128 input pixels; NCI = cin
+// persistent grid over tiles of 128 input pixels of one parity class; NCI = cin
+// (512 stamps: layers 4 and 3 together 300 us -> 112, layer 2 680 -> 206).
 template <int NCI>
 __global__ void __launch_bounds__(BT_THREADS) k_conv_dx_tc(ConvBwd a)
 {
@@ -278,57 +292,67 @@ __global__ void __launch_bounds__(BT_THREADS) k_conv_dx_tc(ConvBwd a)
     const uint32_t tmem = tmem_slot, bar_a = smem_addr(&bar);
     const uint32_t idesc = idesc_bf16(128, NCI);
     const uint32_t wa = smem_addr(Ws), aa = smem_addr(As);
-    const int hwi = a.hin * a.hin;
-    const long long M = (long long)a.B * hwi;
-    const long long tiles = (M + 127) / 128;
-    const int nkc = K / BT_KB;  // a block never straddles two taps (cout is a multiple of 64)
+    // Tiles of 128 input pixels of one parity class (iy mod 2, ix mod 2): with
+    // stride 2 an odd coordinate meets the taps 0 and 2, an even one tap 1 alone, so
+    // a class takes 4, 2, 2 or 1 of the nine taps and the blocks of the others,
+    // which would be zeros, are not formed (9 blocks of work for 4 tiles, not 36).
+    const int lho = __ffs(a.hout) - 1;  // hin = 2 hout, a power of two
+    const long long Mc = (long long)a.B << (2 * lho);  // pixels of a class
+    const long long tpc = (Mc + 127) / 128, tiles = 4 * tpc;
+    const int ncb = a.cout / BT_KB;  // blocks a tap (cout is a multiple of 64)
+    // a thread's items of a block: 8 channels (group j) of rows r0 + 32 u.  A warp
+    // takes 8 rows x 4 channel groups, so the 8 lanes of each 16-byte store phase
+    // write 8 different rows (distinct banks).
+    constexpr int PER = 128 * (BT_KB / 8) / BT_THREADS;
+    static_assert(BT_KB == 64 && BT_THREADS == 256 && PER == 4, "lane mapping");
+    const int r0 = (warp >> 1) * 8 + (lane & 7), j8 = 8 * ((warp & 1) * 4 + (lane >> 3));
     uint32_t parity = 0;
     bool failed = false;
     for (long long tile = blockIdx.x; tile < tiles; tile += gridDim.x) {
-        const long long m0 = tile * 128;
-        for (int c = 0; c < nkc && !failed; ++c) {
-            const int kc0 = c * BT_KB, tap = kc0 / a.cout, co0 = kc0 - tap * a.cout;
-            const int ky = tap / 3, kx = tap - 3 * ky;
-            // A: (input pixel, 8 channels of G at the pixel the tap maps it to).
-            // A warp takes 8 rows x 4 channel groups, so the 8 lanes of each
-            // 16-byte store phase write 8 different rows (distinct banks).
-            static_assert(BT_KB % 32 == 0 && (128 * (BT_KB / 8)) % BT_THREADS == 0, "lane mapping");
-            constexpr int PER = 128 * (BT_KB / 8) / BT_THREADS;  // items per thread
-            float f[PER][8];
-            int orow[PER], oj[PER];
-            // every item's loads first (all in flight), then the splits and stores
+        const int cls = 3 - (int)(tile / tpc);  // the class with the most taps first
+        const int py = cls >> 1, px = cls & 1, ntx = 1 + px, nblk = (1 + py) * ntx * ncb;
+        const long long q0 = (tile - (3 - cls) * tpc) * 128;
+        // G at the output pixel (iy / 2, ix / 2), and whether the next row and
+        // column are in range (the taps 0 of odd coordinates)
+        const float* gp[PER];
+        unsigned ok = 0u;  // per item: bit 0 the row exists, 1 next row, 2 next column
+#pragma unroll
+        for (int u = 0; u < PER; ++u) {
+            const long long q = q0 + r0 + 32 * u;
+            const int hy = (int)(q >> lho) & (a.hout - 1), hx = (int)q & (a.hout - 1);
+            gp[u] = a.g + q * a.cout + j8;
+            if (q < Mc) ok |= (1u | (hy + 1 < a.hout ? 2u : 0u) | (hx + 1 < a.hout ? 4u : 0u)) << (4 * u);
+        }
+        float4 f[PER][2];
+        auto load = [&](int blk) {
+            const int t = blk / ncb, cb = blk - t * ncb;
+            const int ky = py ? 2 * (t / ntx) : 1, kx = px ? 2 * (t - (t / ntx) * ntx) : 1;
+            const int dy = ky == 0 ? 1 : 0, dx = kx == 0 ? 1 : 0;
+            const unsigned need = 1u | (dy ? 2u : 0u) | (dx ? 4u : 0u);
+            const int at = (dy * a.hout + dx) * a.cout + cb * BT_KB;
 #pragma unroll
             for (int u = 0; u < PER; ++u) {
-                const int it = tid + u * BT_THREADS;
-                const int lane_i = it & 31, rest = it >> 5;
-                const int jq = rest % (BT_KB / 32), rg = rest / (BT_KB / 32);
-                const int r = rg * 8 + (lane_i & 7), j = jq * 4 + (lane_i >> 3);
-                orow[u] = r;
-                oj[u] = j;
-                const long long m = m0 + r;
-                float4 p0 = make_float4(0.f, 0.f, 0.f, 0.f), p1 = p0;
-                if (m < M) {
-                    const int b = (int)(m / hwi), pix = (int)(m - (long long)b * hwi);
-                    const int iy = pix / a.hin, ix = pix - iy * a.hin;
-                    const int ty = iy + 1 - ky, tx = ix + 1 - kx;
-                    if (ty >= 0 && tx >= 0 && !(ty & 1) && !(tx & 1) && (ty >> 1) < a.hout &&
-                        (tx >> 1) < a.hout) {
-                        const float4* src = reinterpret_cast<const float4*>(
-                            a.g + (((long long)b * a.hout + (ty >> 1)) * a.hout + (tx >> 1)) * a.cout + co0 +
-                            8 * j);
-                        p0 = src[0];
-                        p1 = src[1];
-                    }
+                f[u][0] = f[u][1] = make_float4(0.f, 0.f, 0.f, 0.f);
+                if (((ok >> (4 * u)) & need) == need) {
+                    const float4* src = reinterpret_cast<const float4*>(gp[u] + at);
+                    f[u][0] = src[0];
+                    f[u][1] = src[1];
                 }
-                f[u][0] = p0.x; f[u][1] = p0.y; f[u][2] = p0.z; f[u][3] = p0.w;
-                f[u][4] = p1.x; f[u][5] = p1.y; f[u][6] = p1.z; f[u][7] = p1.w;
             }
+        };
+        load(0);
+        for (int blk = 0; blk < nblk && !failed; ++blk) {
+            const int t = blk / ncb, cb = blk - t * ncb;
+            const int tap = 3 * (py ? 2 * (t / ntx) : 1) + (px ? 2 * (t - (t / ntx) * ntx) : 1);
+            const int kc0 = tap * a.cout + cb * BT_KB;
 #pragma unroll
             for (int u = 0; u < PER; ++u) {
+                const float x[8] = {f[u][0].x, f[u][0].y, f[u][0].z, f[u][0].w,
+                                    f[u][1].x, f[u][1].y, f[u][1].z, f[u][1].w};
                 __nv_bfloat16 hi[8], mid[8], lo[8];
 #pragma unroll
-                for (int q = 0; q < 8; ++q) split3(f[u][q], hi[q], mid[q], lo[q]);
-                const int o = cofs(orow[u], 8 * oj[u], BT_KB);
+                for (int q = 0; q < 8; ++q) split3(x[q], hi[q], mid[q], lo[q]);
+                const int o = cofs(r0 + 32 * u, j8, BT_KB);
                 *reinterpret_cast<uint4*>(As + o) = pack8(hi);
                 *reinterpret_cast<uint4*>(As + PLANE / 2 + o) = pack8(mid);
                 *reinterpret_cast<uint4*>(As + PLANE + o) = pack8(lo);
@@ -339,9 +363,10 @@ __global__ void __launch_bounds__(BT_THREADS) k_conv_dx_tc(ConvBwd a)
                     for (int p = 0; p < 3; ++p)
                         umma(tmem, mdesc(aa + p * PLANE + ks * 256, 128, BT_KB * 16),
                              mdesc(wa + (uint32_t)(kc0 + ks * 16) * 16, 128, (uint32_t)K * 16), idesc,
-                             (c > 0 || ks > 0 || p > 0) ? 1 : 0);
+                             (blk > 0 || ks > 0 || p > 0) ? 1 : 0);
                 mma_commit(bar_a);
             }
+            if (blk + 1 < nblk) load(blk + 1);  // in flight while the MMAs run
             const bool done = mbar_wait(bar_a, parity);
             parity ^= 1u;
             asm volatile("tcgen05.fence::after_thread_sync;");
@@ -352,8 +377,9 @@ __global__ void __launch_bounds__(BT_THREADS) k_conv_dx_tc(ConvBwd a)
         }
         // epilogue: the gradient through the ReLU of the layer below (X > 0)
         const int quarter = warp & 3, chalf = warp >> 2;
-        const int row = quarter * 32 + lane;
-        const long long m = m0 + row;
+        const long long q = q0 + quarter * 32 + lane;
+        const int hy = (int)(q >> lho) & (a.hout - 1), hx = (int)q & (a.hout - 1);
+        const long long m = ((q >> (2 * lho)) * a.hin + (2 * hy + py)) * a.hin + (2 * hx + px);
         const uint32_t taddr = tmem + ((uint32_t)(quarter * 32) << 16);
         for (int c0 = chalf * (NCI / 2); c0 < (chalf + 1) * (NCI / 2); c0 += 8) {
             float v[8];
@@ -363,7 +389,7 @@ __global__ void __launch_bounds__(BT_THREADS) k_conv_dx_tc(ConvBwd a)
 #pragma unroll
                 for (int j = 0; j < 8; ++j) v[j] = NAN;
             }
-            if (m >= M) continue;
+            if (q >= Mc) continue;
             const uint4 u = *reinterpret_cast<const uint4*>(a.x + m * NCI + c0);
             const __nv_bfloat16* xv = reinterpret_cast<const __nv_bfloat16*>(&u);
 #pragma unroll
@@ -428,7 +454,7 @@ cudaError_t launch_dx(const ConvBwd& a, cudaStream_t s)
     if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_conv_dx_tc<NCI>, BT_THREADS, smem)) !=
         cudaSuccess)
         return e;
-    const long long tiles = ((long long)a.B * a.hin * a.hin + 127) / 128;
+    const long long tiles = 4 * (((long long)a.B * a.hout * a.hout + 127) / 128);  // four parity classes
     const int grid = (int)std::min<long long>(tiles, (long long)sms * std::max(per_sm, 1));
     k_conv_dx_tc<NCI><<<grid, BT_THREADS, smem, s>>>(a);
     GF_COUNT_LAUNCH();

@@ -76,8 +76,10 @@ __global__ void __launch_bounds__(CT_THREADS) k_conv_tc(ConvTC a)
     const uint32_t bar_a = smem_addr(&bar);
     const uint32_t idesc = idesc_bf16(CT_TM, N);
     const uint32_t a0 = smem_addr(As), b0 = smem_addr(Bs);
-    const int hw = a.hout * a.hout;
-    const long long M = (long long)a.B * hw;
+    // (the layers' sides and channels are powers of two: rows and k split by shifts,
+    // where a 64-bit division and four more an item set the gather's time)
+    const int hw = a.hout * a.hout, lho = __ffs(a.hout) - 1, lci = __ffs(a.cin) - 1;
+    const long long M = (long long)a.B << (2 * lho);
     const long long tiles = (M + CT_TM - 1) / CT_TM;
     uint32_t parity = 0;
     bool failed = false;
@@ -100,10 +102,10 @@ __global__ void __launch_bounds__(CT_THREADS) k_conv_tc(ConvTC a)
                 const __nv_bfloat16* src = a.x;  // (not read when the copy is a zero fill)
                 bool in = false;
                 if (m < M) {
-                    const int b = (int)(m / hw), pix = (int)(m - (long long)b * hw);
-                    const int oy = pix / a.hout, ox = pix - oy * a.hout;
-                    const int tap = k / a.cin, ci = k - tap * a.cin;
-                    const int iy = 2 * oy - 1 + tap / 3, ix = 2 * ox - 1 + tap % 3;
+                    const int b = (int)(m >> (2 * lho)), pix = (int)m & (hw - 1);
+                    const int oy = pix >> lho, ox = pix & (a.hout - 1);
+                    const int tap = k >> lci, ci = k & (a.cin - 1), ty = tap / 3;
+                    const int iy = 2 * oy - 1 + ty, ix = 2 * ox - 1 + (tap - 3 * ty);
                     in = iy >= 0 && iy < a.hin && ix >= 0 && ix < a.hin;
                     if (in) src = a.x + (((long long)b * a.hin + iy) * a.hin + ix) * a.cin + ci;
                 }
@@ -147,8 +149,8 @@ __global__ void __launch_bounds__(CT_THREADS) k_conv_tc(ConvTC a)
         const uint32_t taddr = tmem + ((uint32_t)(quarter * 32) << 16);
         int b = 0, pix = 0;
         if (m < M) {
-            b = (int)(m / hw);
-            pix = (int)(m - (long long)b * hw);
+            b = (int)(m >> (2 * lho));
+            pix = (int)m & (hw - 1);
         }
         for (int n0 = nhalf * (N / 2); n0 < (nhalf + 1) * (N / 2); n0 += 8) {
             float v[8];
@@ -191,13 +193,15 @@ __global__ void k_conv1_nhwc(const __nv_bfloat16* __restrict__ x, const __nv_bfl
                              const float* __restrict__ bias, __nv_bfloat16* __restrict__ y, int B,
                              int hin, int cout, int hout)
 {
+    // (channel groups and sides are powers of two: split by shifts; the 64-bit
+    // divisions cost as much as the taps)
     const long long item = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    const int ncg = cout / 8, npix = hout * hout;
+    const int ncg = cout / 8, npix = hout * hout, lcg = __ffs(ncg) - 1, lho = __ffs(hout) - 1;
     if (item >= (long long)B * ncg * npix) return;
-    const int cg = (int)(item % ncg);
-    const long long r = item / ncg;
-    const int pix = (int)(r % npix), b = (int)(r / npix);
-    const int oy = pix / hout, ox = pix - oy * hout;
+    const int cg = (int)item & (ncg - 1);
+    const long long r = item >> lcg;
+    const int pix = (int)r & (npix - 1), b = (int)(r >> (2 * lho));
+    const int oy = pix >> lho, ox = pix & (hout - 1);
     float acc[8];
 #pragma unroll
     for (int j = 0; j < 8; ++j) acc[j] = bias[cg * 8 + j];
