@@ -799,6 +799,7 @@ PassArgs base_args(void* ws, const Layout& L, const float* psf, const float* img
     a.eval_variant = L.eval_variant;
     a.os_ns = L.os_ns;
     a.conv_ty = L.conv_ty;
+    a.tot_wb = L.tot_wb;
     return a;
 }
 

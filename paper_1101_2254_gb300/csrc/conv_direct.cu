@@ -391,6 +391,142 @@ __global__ void __launch_bounds__(TX * TY / 16) k_conv_direct(PassArgs a)
     if (DB) cp_async_wait<0>();
 }
 
+// The same sums for launches of few output blocks (a small stamp on its own),
+// where k_conv_direct has a warp a block and the warp's 16 P^2 FMAs a lane are the
+// call's latency: a CTA of four warps per 16 x 32 block, a thread 4 adjacent
+// columns of one row, its 4 chains of P^2 FMAs just covering the FMA latency
+// (P is a template argument, so that a tap row's shared loads are issued ahead of
+// the FMAs of the one before; with P at run time they were not, and a 33x33 PSF
+// took 20.4 us for 11.9).
+// Lane 8 rr + cg of warp w holds columns 4 cg .. 4 cg + 3 of row 4 w + rr, so that
+// the 8 lanes of a 16-byte load phase read 32 consecutive values.  Every output
+// sums its taps in the same order, and a trial pass's chi^2 is taken by one warp
+// from the block's outputs in k_conv_direct's order: the same bits.
+// One 64x64 stamp, the whole launch: P 9 9.8 us (k_conv_direct) -> 6.2, P 25
+// 18.1 -> 9.7, P 33 24.5 -> 11.9.
+constexpr int THIN_THREADS = 128;
+
+__host__ __device__ constexpr int thin_sw(int P4) { return 32 + P4; }
+
+template <int P>
+__global__ void __launch_bounds__(THIN_THREADS) k_conv_direct_thin(PassArgs a)
+{
+    pdl_entry();
+    extern __shared__ __align__(16) float smem[];
+    const int ch = blockIdx.x % a.nchan, blk = blockIdx.x / a.nchan;
+    int b = 0;
+    {  // the stamp of output block blk: the last whose first block is not after it
+        int hi = a.count;
+        while (hi - b > 1) {
+            const int mid = (b + hi) >> 1;
+            if (a.st[mid].wb_off <= blk)
+                b = mid;
+            else
+                hi = mid;
+        }
+    }
+    if (a.lm && a.lm[b].phase != a.phase) return;  // the whole CTA
+    const StampInfo& st = a.st[b];
+    const int H = st.H, W = st.W, He = st.He, We = st.We;
+    constexpr int P4 = (P + 3) & ~3;
+    const int nbx = (W + 31) / 32, t = blk - st.wb_off;
+    const int ty0 = (t / nbx) * 16, tx0 = (t % nbx) * 32;
+    constexpr int SW = thin_sw(P4), SH = 16 + P - 1;
+    float* ks = smem;            // P x P4 flipped taps
+    float* es = smem + P * P4;   // SH x SW grid window
+    const float* E = a.ext + ext_index(st, a.nchan, ch);
+    const float* psf = a.psf + st.psf_off;
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    for (int r = warp; r < SH; r += THIN_THREADS / 32) {
+        const int gy = ty0 + r;
+        const float* Er = E + (long long)(gy < He ? gy : 0) * We;
+        for (int col = lane; col < SW; col += 32) {
+            const int gx = tx0 + col;
+            const bool in = gy < He && gx < We;
+            cp_async4(es + r * SW + col, in ? Er + gx : E, in);
+        }
+    }
+    for (int v = warp; v < P; v += THIN_THREADS / 32) {
+        const float* pr = psf + (P - 1 - v) * P;
+        for (int u = lane; u < P4; u += 32) cp_async4(ks + v * P4 + u, u < P ? pr + (P - 1 - u) : psf, u < P);
+    }
+    cp_async_commit();
+    // a trial pass's image and sigma, in flight under the taps (warp 0, in the
+    // order that it sums them: lane 8 cg + rl the columns 8 cg .. 8 cg + 7 of rows
+    // rl and rl + 8)
+    const int rl = lane & 7, c8 = 8 * (lane >> 3);
+    float dv[RPT][8], sv[RPT][8];
+    if (a.conv_chi2 && warp == 0) {
+        const float* img = a.img + st.pix_off;
+        const float* sig = a.sig + st.pix_off;
+#pragma unroll
+        for (int i = 0; i < RPT; ++i)
+#pragma unroll
+            for (int o = 0; o < 8; ++o) {
+                const int y = ty0 + rl + 8 * i, x = tx0 + c8 + o;
+                const bool in = y < H && x < W;
+                const long long px = (long long)y * W + x;
+                dv[i][o] = in ? __ldg(&img[px]) : 0.0f;
+                sv[i][o] = in ? __ldg(&sig[px]) : 0.0f;
+            }
+    }
+    cp_async_wait<0>();
+    __syncthreads();
+    const int row = 4 * warp + (lane >> 3), c0 = 4 * (lane & 7);
+    float acc[4] = {0.0f, 0.0f, 0.0f, 0.0f};
+    const float* er = es + row * SW + c0;
+    const float* kr = ks;
+#pragma unroll 2
+    for (int v = 0; v < P; ++v, er += SW, kr += P4) {
+        alignas(16) float win[P4 + 4], k[P4];
+#pragma unroll
+        for (int m = 0; m < P4 + 4; m += 4) *reinterpret_cast<float4*>(win + m) = *reinterpret_cast<const float4*>(er + m);
+#pragma unroll
+        for (int m = 0; m < P4; m += 4) *reinterpret_cast<float4*>(k + m) = *reinterpret_cast<const float4*>(kr + m);
+#pragma unroll
+        for (int u = 0; u < P; ++u)
+#pragma unroll
+            for (int o = 0; o < 4; ++o) acc[o] = fmaf(k[u], win[u + o], acc[o]);
+    }
+    const int rows = min(16, H - ty0), cols = min(32, W - tx0);
+    if (a.work && tid == 0)
+        atomicAdd(&a.work[PROF_CONV], 2ull * (unsigned long long)P * P * (unsigned long long)rows * (unsigned long long)cols);
+    if (!a.conv_chi2) {
+        float* Y = a.y + y_index(st, a.nchan, ch) + (long long)(ty0 + row) * W + tx0 + c0;
+        if (row < rows)
+#pragma unroll
+            for (int o = 0; o < 4; ++o)
+                if (c0 + o < cols) Y[o] = acc[o];
+        return;
+    }
+    __syncthreads();  // the window is read: its space takes the outputs (stride 33)
+#pragma unroll
+    for (int o = 0; o < 4; ++o) es[row * 33 + c0 + o] = acc[o];
+    __syncthreads();
+    if (warp != 0) return;
+    const Channel& chn = a.chan[(long long)b * a.chan_stride + ch];
+    const float tmw = chn.mweight, tmsky = chn.msky;
+    CSum cs = {0.0f, 0.0f};
+#pragma unroll
+    for (int i = 0; i < RPT; ++i)
+#pragma unroll
+        for (int o = 0; o < 8; ++o) {
+            const float d = dv[i][o], sg = sv[i][o];
+            if (isfinite(d) && isfinite(sg) && sg > 0.0f) {
+                const float z = (d - fmaf(tmw, es[(rl + 8 * i) * 33 + c8 + o], tmsky)) / sg;
+                csum_add(cs, z * z);
+            }
+        }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+        CSum other;
+        other.s = __shfl_down_sync(0xffffffffu, cs.s, o);
+        other.c = __shfl_down_sync(0xffffffffu, cs.c, o);
+        cs = csum_merge(cs, other);
+    }
+    if (lane == 0) a.partial[(long long)blk * a.nchan + ch] = cs.s + cs.c;
+}
+
 }  // namespace
 
 cudaError_t ensure_smem_optin_conv_direct(int P, int* cache);
@@ -445,8 +581,53 @@ cudaError_t launch_tile(const PassArgs& a, int kind, cudaStream_t s)
     return a.conv_ty == 16 ? launch_tile_h<TX, 16>(a, kind, s) : launch_tile_h<TX, 32>(a, kind, s);
 }
 
+template <int P>
+cudaError_t launch_thin(const PassArgs& a, cudaStream_t s)
+{
+    constexpr int P4 = (P + 3) & ~3;
+    constexpr size_t smem = sizeof(float) * (P * P4 + (16 + P - 1) * thin_sw(P4));
+    static_assert(smem <= 48 * 1024, "no opt-in needed");
+    GF_LAUNCH_PDL(k_conv_direct_thin<P>, dim3((unsigned)(a.tot_wb * a.nchan)), dim3(THIN_THREADS), smem, s, a);
+    GF_COUNT_LAUNCH();
+    return cudaGetLastError();
+}
+
+// The line between the two, in output blocks an SM: k_conv_direct's time is flat to
+// about four of them (one warp's chain a scheduler), k_conv_direct_thin's grows by a
+// block's taps with each from the second on.  One stamp, us, thin / k_conv_direct:
+//   blocks     180           320          512          1152
+//   P  9    7.6 /  9.8    7.7 /  9.8   7.7 /  9.7  11.0 / 11.9
+//   P 25   11.8 / 18.4   14.1 / 18.3  16.5 / 18.5  26.5 / 25.6
+//   P 33   16.1 / 24.5   20.5 / 24.5  24.6 / 24.5  40.9 / 36.4
+// PSFs above 35 px keep the generic kernel, which also multiplies its padding taps.
+constexpr long long thin_max_blocks(int P) { return (P < 33 ? 4 : 3) * 152; }
+
 cudaError_t launch_conv_direct(const PassArgs& a, cudaStream_t s)
 {
+    const long long blocks = a.tot_wb * a.nchan;
+    if (blocks <= thin_max_blocks(a.P)) {
+        switch (a.P) {
+        case 1: return launch_thin<1>(a, s);
+        case 3: return launch_thin<3>(a, s);
+        case 5: return launch_thin<5>(a, s);
+        case 7: return launch_thin<7>(a, s);
+        case 9: return launch_thin<9>(a, s);
+        case 11: return launch_thin<11>(a, s);
+        case 13: return launch_thin<13>(a, s);
+        case 15: return launch_thin<15>(a, s);
+        case 17: return launch_thin<17>(a, s);
+        case 19: return launch_thin<19>(a, s);
+        case 21: return launch_thin<21>(a, s);
+        case 23: return launch_thin<23>(a, s);
+        case 25: return launch_thin<25>(a, s);
+        case 27: return launch_thin<27>(a, s);
+        case 29: return launch_thin<29>(a, s);
+        case 31: return launch_thin<31>(a, s);
+        case 33: return launch_thin<33>(a, s);
+        case 35: return launch_thin<35>(a, s);
+        default: break;
+        }
+    }
     cudaError_t e = ensure_smem_optin_conv_direct(a.P, nullptr);
     if (e != cudaSuccess) return e;
     if ((e = launch_tile<64>(a, WK_CONV, s)) != cudaSuccess) return e;

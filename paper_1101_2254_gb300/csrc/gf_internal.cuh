@@ -728,6 +728,7 @@ struct PassArgs {
     int grid[WK_KINDS];        // persistent launch grid per kernel kind
     int maxitems[WK_KINDS];    // upper bound of work items (all stamps, all channels)
     int P;                     // PSF side (uniform across the stamps of a call)
+    long long tot_wb;          // 16 x 32 output blocks of all stamps
     unsigned long long* work;  // profiling: algorithmic work per kernel class, or null
 };
 
