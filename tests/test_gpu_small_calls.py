@@ -60,3 +60,29 @@ def test_few_block_fits_take_the_steps_of_many(gf, P, H, W):
     (p1, r1), (pn, rn) = fits
     assert (np.asarray(pn) == np.asarray(p1)[0]).all()
     assert (np.asarray(rn.chi2) == np.asarray(r1.chi2)[0]).all()
+
+
+def test_nan_amplitude_is_nan_everywhere(gf):
+    # with n inside the table of b_n, above it (solved for otherwise) and below zero;
+    # the stamp beside them keeps its bits
+    kinds, H, W, P = [synth.SERSIC, synth.SKY], 20, 33, 5
+    rng = np.random.default_rng(4)
+    p = np.tile(synth.random_params(kinds, rng, H, W), (5, 1))
+    p[1:, 4] = 3.0, 12.0, -1.0, 12.0
+    p[1:4, 2] = np.nan
+    img = torch.as_tensor(rng.standard_normal(5 * H * W).astype(np.float32)).cuda()
+    psf = torch.as_tensor(np.tile(synth.random_psf(P, 1).astype(np.float32).ravel(), 5)).cuda()
+    d = gf.make_desc(1, 1, P, kinds, 1, 0)
+
+    def run(rows):
+        n = H * W
+        x2, m = gf.evaluate_batch(d, gf.make_batch([H] * len(rows), [W] * len(rows), psf_size=P), p[rows],
+                                  torch.cat([img[r * n:(r + 1) * n] for r in rows]),
+                                  torch.ones(len(rows) * n, device="cuda"), psf[:len(rows) * P * P], want_model=True)
+        return x2.cpu().numpy(), m.cpu().numpy().reshape(len(rows), n)
+
+    x2, m = run([0, 1, 2, 3, 4])
+    assert np.isnan(m[1:4]).all() and np.isfinite(m[[0, 4]]).all() and np.isfinite(x2[[0, 4]]).all()
+    for k in (0, 4):
+        y2, my = run([k])
+        assert y2[0] == x2[k] and np.array_equal(my[0], m[k])
