@@ -10,7 +10,7 @@ struct FFTArgs {
     int Nx, Ny;          // padded transform sizes (Nx even)
     int cpc;             // spectrum columns per CTA in the column pass
     int small;           // 1: one CTA per transform (Nx, Ny in 32 x {3, 4, 5});
-                         // hhat then holds each column in warp-FFT order
+                         // hhat then lies in the order phase B reads it
     int toy, tox;        // small: outputs of a tile
     int one_tile;        // small: every stamp is one tile (the FFT method)
     FFTPlan px, py;
