@@ -130,7 +130,7 @@ typedef enum {
                            (gf_eval_batch, gf_eval_batch_dev, gf_lm_fit_batch,
                            gf_lm_fit_multistart) take P from 23 to 39 through the FFT's
                            one-CTA transform instead, in overlapping tiles, for stamps of
-                           any sizes.  (Stamps of one size whose extended grid is at most
+                           any sizes (evaluations of few pixels stay direct).  (Stamps of one size whose extended grid is at most
                            160 x 160 are one transform each under GF_CONV_FFT: name it
                            there.) */
     GF_CONV_DIRECT = 1, /* tiled direct sum, PSF and halo tile in shared memory */
@@ -405,7 +405,9 @@ gf_status gf_lm_fit_multistart(const gf_desc* d, const gf_batch* b, int starts,
  * on the whole batch, then the widths again under the chosen pair (12 shapes
  * per odd class, 6 per even one).  It synchronises the stream, must not run
  * under stream capture, and needs a workspace of gf_workspace_size_batch()
- * bytes.  It does nothing for Fourier-space convolution. */
+ * bytes.  It does nothing for Fourier-space convolution; under
+ * GF_CONV_AUTO the batched calls take P from 23 to 39 through the FFT's tiles,
+ * which have no shape to tune. */
 gf_status gf_autotune(const gf_desc* d, const gf_batch* b, const float* psf_dev, void* ws,
                       size_t ws_bytes, gf_stream stream);
 /* The tile width (64 or 32) the current device uses for PSF side P and width W. */

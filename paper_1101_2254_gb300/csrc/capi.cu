@@ -129,18 +129,30 @@ int comp_slots(int kind)
 // direct / tiled):
 //   400 stamps of 32-256 px   P 21: 187 / 130   25: 236 / 134   33: 424 / 135   39: 676 / 199
 //   400 stamps of 48-64 px    P 21:  53 / 58    25:  67 / 57    33:  98 / 68    39: 176 / 85
-// and a fit makes the spectra once.  The line depends on P alone, so that a
-// stamp's result does not depend on the batch around it; single-stamp calls,
-// where the set-up's launches count, keep the direct sum.
+// and a fit makes the spectra once.  A fit's line depends on P alone, so that a
+// stamp's fit does not depend on the batch around it; single-stamp calls and small
+// evaluations, where the set-up's launches count, keep the direct sum.
 constexpr int CONV_TILED = 100;
 constexpr int TILED_MIN_PSF = 23;
 
-// d as a batched call resolves it (d is checked)
-gf_desc batch_desc(const gf_desc* d)
+// d as a batched call resolves it (d is checked).  An evaluation of few output
+// blocks (16 x 32) stays with the direct sum: the tiles' twiddles and PSF spectra are
+// launches of their own, made for one pass, where a fit makes them once for all.
+// gf_eval_batch of 64x64 stamps, us, direct / tiled (* the choice):
+//   blocks     64         256        480        800        1600
+//   P 23      45* / -     47* / -     51* / -     65* / 77    76* / 89
+//   P 33      54* / -     60* / -     86  / 76*   85  / 68*  100  / 93*
+gf_desc batch_desc(const gf_desc* d, const gf_batch* eval = nullptr)
 {
     gf_desc e = *d;
-    if (e.conv_method == GF_CONV_AUTO && e.psf_size >= TILED_MIN_PSF && e.psf_size < GF_AUTO_FFT_PSF)
-        e.conv_method = CONV_TILED;
+    if (e.conv_method != GF_CONV_AUTO || e.psf_size < TILED_MIN_PSF || e.psf_size >= GF_AUTO_FFT_PSF) return e;
+    if (eval) {
+        long long blocks = 0;
+        for (int i = 0; i < eval->count; ++i)
+            blocks += (((long long)eval->H[i] + 15) / 16) * (((long long)eval->W[i] + 31) / 32);
+        if (blocks <= (e.psf_size < 33 ? 12 * 152 : conv_thin_max_blocks(e.psf_size))) return e;
+    }
+    e.conv_method = CONV_TILED;
     return e;
 }
 
@@ -1364,7 +1376,7 @@ size_t gf_workspace_size_eval_batch(const gf_desc* d, const gf_batch* b)
 {
     if (!b || b->count < 1 || !b->H || !b->W) return 0;
     if (check_structure(d) != GF_OK) return 0;
-    const gf_desc db = batch_desc(d);
+    const gf_desc db = batch_desc(d, b);
     d = &db;
     for (int i = 0; i < b->count; ++i)
         if (check_stamp(d, b->H[i], b->W[i]) != GF_OK) return 0;
@@ -1546,9 +1558,9 @@ static gf_status eval_batch_impl(const gf_desc* d, const gf_batch* b, const doub
 {
     gf_status r = check_structure(d);
     if (r != GF_OK) return r;
-    const gf_desc db = batch_desc(d);
-    d = &db;
     if (!b || b->count < 1 || !b->H || !b->W) return fail(GF_EINVAL, "bad batch");
+    const gf_desc db = batch_desc(d, b);
+    d = &db;
     for (int i = 0; i < b->count; ++i)
         if ((r = check_stamp(d, b->H[i], b->W[i])) != GF_OK) return r;
     if ((r = check_fft(d, b->count, b->H, b->W)) != GF_OK) return r;
@@ -1833,7 +1845,7 @@ gf_status gf_autotune(const gf_desc* d, const gf_batch* b, const float* psf, voi
         if ((rr = upload(ws, make_blob(pl, S, nullptr), s)) != GF_OK) return rr;
         PassArgs a = jac_args(ws, pl.L, base_args(ws, pl.L, psf, nullptr, nullptr, P));
         auto launch = [&]() {
-            return tile_w > 0 ? launch_conv_direct_width(a, tile_w, s) : launch_conv_direct(a, s);
+            return launch_conv_direct_width(a, tile_w, s);
         };
         if (cudaMemsetAsync(a.ext, 0, sizeof(float) * (size_t)pl.L.nchan *
                                           (pl.st.back().ext1_off +

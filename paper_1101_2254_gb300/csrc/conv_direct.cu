@@ -600,12 +600,12 @@ cudaError_t launch_thin(const PassArgs& a, cudaStream_t s)
 //   P 25   11.8 / 18.4   14.1 / 18.3  16.5 / 18.5  26.5 / 25.6
 //   P 33   16.1 / 24.5   20.5 / 24.5  24.6 / 24.5  40.9 / 36.4
 // PSFs above 35 px keep the generic kernel, which also multiplies its padding taps.
-constexpr long long thin_max_blocks(int P) { return (P < 33 ? 4 : 3) * 152; }
+long long conv_thin_max_blocks(int P) { return P > 35 ? 0 : (P < 33 ? 4 : 3) * 152; }
 
 cudaError_t launch_conv_direct(const PassArgs& a, cudaStream_t s)
 {
     const long long blocks = a.tot_wb * a.nchan;
-    if (blocks <= thin_max_blocks(a.P)) {
+    if (blocks <= conv_thin_max_blocks(a.P)) {
         switch (a.P) {
         case 1: return launch_thin<1>(a, s);
         case 3: return launch_thin<3>(a, s);
@@ -628,18 +628,17 @@ cudaError_t launch_conv_direct(const PassArgs& a, cudaStream_t s)
         default: break;
         }
     }
-    cudaError_t e = ensure_smem_optin_conv_direct(a.P, nullptr);
-    if (e != cudaSuccess) return e;
-    if ((e = launch_tile<64>(a, WK_CONV, s)) != cudaSuccess) return e;
-    return launch_tile<32>(a, WK_CONV32, s);
+    return launch_conv_direct_width(a, 0, s);
 }
 
-// launch one tile width alone (the tuner times the two against each other)
+// k_conv_direct whatever the blocks, for one tile width alone or both (0): the
+// tuner times its widths and shapes against each other
 cudaError_t launch_conv_direct_width(const PassArgs& a, int tile_w, cudaStream_t s)
 {
     cudaError_t e = ensure_smem_optin_conv_direct(a.P, nullptr);
     if (e != cudaSuccess) return e;
-    return tile_w == 64 ? launch_tile<64>(a, WK_CONV, s) : launch_tile<32>(a, WK_CONV32, s);
+    if (tile_w != 32 && (e = launch_tile<64>(a, WK_CONV, s)) != cudaSuccess) return e;
+    return tile_w != 64 ? launch_tile<32>(a, WK_CONV32, s) : cudaSuccess;
 }
 
 // The shared-memory opt-in of the four tile shapes' kernels for a P x P PSF,

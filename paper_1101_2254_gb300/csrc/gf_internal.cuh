@@ -786,6 +786,7 @@ cudaError_t launch_fma_peak(int fp64, int grid, int iters, void* sink, cudaStrea
 cudaError_t launch_model(const PassArgs& a, cudaStream_t s);
 cudaError_t launch_conv_direct(const PassArgs& a, cudaStream_t s);
 cudaError_t launch_conv_direct_width(const PassArgs& a, int tile_w, cudaStream_t s);
+long long conv_thin_max_blocks(int P);  // output blocks x channels up to which k_conv_direct_thin runs
 cudaError_t launch_reduce_jac(const PassArgs& a, cudaStream_t s);
 cudaError_t launch_reduce_chi2(const PassArgs& a, cudaStream_t s);
 // chi^2 partials of each channel as its own model (the rungs of a trial pass)

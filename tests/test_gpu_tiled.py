@@ -13,7 +13,7 @@ from paper_1101_2254_gb300 import synth
 pytestmark = pytest.mark.gpu
 torch = pytest.importorskip("torch")
 
-SIZES = [(64, 64), (65, 63), (1, 1), (3, 129), (128, 65), (80, 97), (16, 32), (17, 33), (200, 40), (31, 161)]
+SIZES = [(64, 64), (65, 63), (1, 1), (3, 129), (128, 65), (80, 97), (16, 32), (17, 33), (200, 40), (31, 161)] * 17  # 1887 blocks: fewer would take the direct sum
 KINDS = [synth.SERSIC, synth.EXPDISK, synth.SKY]
 
 
