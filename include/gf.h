@@ -126,14 +126,18 @@ typedef enum {
 } gf_comp_kind;
 
 typedef enum {
-    GF_CONV_AUTO = 0,   /* direct for P < GF_AUTO_FFT_PSF, else FFT.  The batched calls
-                           (gf_eval_batch, gf_eval_batch_dev, gf_lm_fit_batch,
-                           gf_lm_fit_multistart) take P from 23 to 39 through the FFT's
-                           one-CTA transform instead, in overlapping tiles, for stamps of
-                           any sizes (evaluations of few pixels stay direct).  (Stamps of one size whose extended grid is at most
-                           160 x 160 are one transform each under GF_CONV_FFT: name it
-                           there.) */
-    GF_CONV_DIRECT = 1, /* tiled direct sum, PSF and halo tile in shared memory */
+    GF_CONV_AUTO = 0,   /* direct for P < GF_AUTO_FFT_PSF, else FFT.  From P = 23 the
+                           direct sum adds each tap row apart, which keeps its error
+                           below 6e-7 of every pixel.  The choice depends on P alone: a
+                           stamp gives the same bits in every call and every batch.
+                           (For extended grids up to 160 x 160 the FFT is one CTA per
+                           transform and overtakes the direct sum from about P = 15 on
+                           64x64 and 96x96 stamps, P = 33 on 32x32: name GF_CONV_FFT
+                           there, if round-off of 2e-7 of the brightest pixel in every
+                           pixel will do: on a faint sky beside a bright compact source
+                           that can be a hundredth of the pixel.) */
+    GF_CONV_DIRECT = 1, /* tiled direct sum, PSF and halo tile in shared memory; the P^2
+                           taps of a pixel in one chain (error to 1e-5 of it at P = 39) */
     GF_CONV_FFT = 2,    /* shared-memory mixed-radix FFT, 2^a 3^b 5^c sizes up to 4096;
                            the stamps of one call must share H and W.  Extended grids
                            up to 160 x 160 are padded to Nx, Ny in {96, 128, 160} and
@@ -405,9 +409,7 @@ gf_status gf_lm_fit_multistart(const gf_desc* d, const gf_batch* b, int starts,
  * on the whole batch, then the widths again under the chosen pair (12 shapes
  * per odd class, 6 per even one).  It synchronises the stream, must not run
  * under stream capture, and needs a workspace of gf_workspace_size_batch()
- * bytes.  It does nothing for Fourier-space convolution; under
- * GF_CONV_AUTO the batched calls take P from 23 to 39 through the FFT's tiles,
- * which have no shape to tune. */
+ * bytes.  It does nothing for Fourier-space convolution. */
 gf_status gf_autotune(const gf_desc* d, const gf_batch* b, const float* psf_dev, void* ws,
                       size_t ws_bytes, gf_stream stream);
 /* The tile width (64 or 32) the current device uses for PSF side P and width W. */

@@ -121,39 +121,25 @@ int comp_slots(int kind)
     }
 }
 
-// The batched calls' convolution under GF_CONV_AUTO for PSF sides in
-// [TILED_MIN_PSF, GF_AUTO_FFT_PSF): overlap-save tiles through the one-CTA
-// transform (conv_fft.cu), for stamps of any sizes.  Not a value that a caller
-// may name.  The direct sum costs P^2 FMAs an output, a tile's transforms the
-// same for every P.  Convolution of one evaluation, PSF spectra included (us,
-// direct / tiled):
-//   400 stamps of 32-256 px   P 21: 187 / 130   25: 236 / 134   33: 424 / 135   39: 676 / 199
-//   400 stamps of 48-64 px    P 21:  53 / 58    25:  67 / 57    33:  98 / 68    39: 176 / 85
-// and a fit makes the spectra once.  A fit's line depends on P alone, so that a
-// stamp's fit does not depend on the batch around it; single-stamp calls and small
-// evaluations, where the set-up's launches count, keep the direct sum.
-constexpr int CONV_TILED = 100;
-constexpr int TILED_MIN_PSF = 23;
+// From this PSF side on the automatic method's direct sum adds its taps row by row
+// (conv_direct.cu, which has the errors of both): the one chain's round-off grows
+// with its P^2 links, to 1e-5 of a pixel at 39, and the rows' stays at a few 2^-24.
+// Below, and where the caller names GF_CONV_DIRECT, the sum is the one chain.  The
+// rule reads P alone, so that a stamp's numbers are the same bits in every call
+// and in every batch.
+// It is not a Fourier method because a float32 transform's round-off is that of the
+// grid's brightest pixel: 2e-3 to 4e-1 of the faint pixels around a galaxy of flux
+// 1e5 to 1e7, where chi^2 counts them with a sigma as small as they are.  That costs
+// speed, which a caller who can afford the error has by naming GF_CONV_FFT.
+// Convolution of one pass of a fit, us a launch, one chain / tap rows / overlap-save
+// tiles of a float32 FFT, which stood here for batched calls: 2,000 stamps of 64x64,
+// P 25 577 / 505 / 231, P 33 942 / 835 / 240; 500 of 100x100, P 37 1,664 / 1,094 /
+// 350; one of 128x128, P 33 21.6 / 12.7 / 18.7.
+constexpr int CONV_ROWS_MIN_PSF = 23;
 
-// d as a batched call resolves it (d is checked).  An evaluation of few output
-// blocks (16 x 32) stays with the direct sum: the tiles' twiddles and PSF spectra are
-// launches of their own, made for one pass, where a fit makes them once for all.
-// gf_eval_batch of 64x64 stamps, us, direct / tiled (* the choice):
-//   blocks     64         256        480        800        1600
-//   P 23      45* / -     47* / -     51* / -     65* / 77    76* / 89
-//   P 33      54* / -     60* / -     86  / 76*   85  / 68*  100  / 93*
-gf_desc batch_desc(const gf_desc* d, const gf_batch* eval = nullptr)
+bool conv_rows(const gf_desc* d)
 {
-    gf_desc e = *d;
-    if (e.conv_method != GF_CONV_AUTO || e.psf_size < TILED_MIN_PSF || e.psf_size >= GF_AUTO_FFT_PSF) return e;
-    if (eval) {
-        long long blocks = 0;
-        for (int i = 0; i < eval->count; ++i)
-            blocks += (((long long)eval->H[i] + 15) / 16) * (((long long)eval->W[i] + 31) / 32);
-        if (blocks <= (e.psf_size < 33 ? 12 * 152 : conv_thin_max_blocks(e.psf_size))) return e;
-    }
-    e.conv_method = CONV_TILED;
-    return e;
+    return d->conv_method == GF_CONV_AUTO && d->psf_size >= CONV_ROWS_MIN_PSF && d->psf_size < GF_AUTO_FFT_PSF;
 }
 
 int resolve_method(const gf_desc* d)
@@ -521,6 +507,7 @@ struct Layout {
     long long tot_wb;  // 16 x 32 output blocks of all stamps (the fused trial chi^2's partials)
     long long max_wb;  // ... and the most of one stamp
     int conv_ty, conv_cap;  // direct convolution: tile height, persistent CTAs per SM
+    int conv_rows;          // and whether its tap rows are summed apart
     int eval_variant;  // the model kernels' evaluator: 0 Sersic / disk / Gaussian,
                        // 1 with Moffat, 2 with King, Nuker or point sources
     int os_ns;         // sub-samples per oversampled pixel (os_factor^2; 1 without a block)
@@ -530,10 +517,10 @@ struct Plan {
     Layout L;
     std::vector<StampInfo> st;
     std::vector<int> pre;  // 4 * (count + 1): model, os, conv, red
-    int method;            // GF_CONV_DIRECT, GF_CONV_FFT, CONV_TILED or GF_CONV_DFT_TC
-    int Nx = 0, Ny = 0, cpc = 0;  // FFT geometry (methods FFT and tiled)
+    int method;            // GF_CONV_DIRECT, GF_CONV_FFT or GF_CONV_DFT_TC
+    int Nx = 0, Ny = 0, cpc = 0;  // FFT geometry (method FFT)
     int small = 0;         // FFT: one CTA per transform (Nx, Ny in 32 x {3, 4, 5})
-    int toy = 0, tox = 0;  // small: outputs of a tile (the stamp's own size, method FFT)
+    int toy = 0, tox = 0;  // small: outputs of a transform (the stamp's size)
     DftFactor fx, fy;      // DFT geometry (method DFT_TC)
 };
 
@@ -599,12 +586,6 @@ void plan_batch(const gf_desc* d, const Structure& S, int count, const int* H, c
         pl->toy = s0.H;
         pl->tox = s0.W;
     }
-    if (pl->method == CONV_TILED) {
-        pl->Nx = pl->Ny = fft_tile_len(P);
-        pl->small = 1;
-        pl->toy = fft_tile_toy(P);
-        pl->tox = fft_tile_tox(P);
-    }
     if (pl->small)  // the convolution's work items are the transform's tiles
         for (int b = 0; b < count; ++b) {
             const StampInfo& s = pl->st[b];
@@ -617,6 +598,7 @@ void plan_batch(const gf_desc* d, const Structure& S, int count, const int* H, c
     L.max_wb = max_wb;
     L.tot_wb = wb;
     L.conv_ty = shape.ty;
+    L.conv_rows = conv_rows(d);
     L.conv_cap = shape.ctas_per_sm;
     L.count = count;
     L.nchan = S.nchan;
@@ -697,7 +679,7 @@ void plan_batch(const gf_desc* d, const Structure& S, int count, const int* H, c
         L.wl_blk = o;
         o += al(sizeof(int) * (size_t)worklist_blocks(count) * (1 + WK_KINDS));
     }
-    if (pl->method == GF_CONV_FFT || pl->method == CONV_TILED) {
+    if (pl->method == GF_CONV_FFT) {
         const StampInfo& s0 = pl->st[0];
         if (!pl->small) {
             pl->Nx = fft_len(s0.We, true);
@@ -712,7 +694,7 @@ void plan_batch(const gf_desc* d, const Structure& S, int count, const int* H, c
         L.hhat = o;
         o += al(sizeof(float2) * (size_t)count * pl->Ny * Kx);
         L.psfgrid = o;
-        if (pl->method == GF_CONV_FFT) o += al(sizeof(float) * (size_t)count * pl->Ny * pl->Nx);
+        o += al(sizeof(float) * (size_t)count * pl->Ny * pl->Nx);
         const size_t spec_rows = pl->small ? 0 : (size_t)s0.He * Kx;
         if (need & (NEED_JAC | NEED_LM)) {
             L.spec_jac = o;
@@ -811,6 +793,7 @@ PassArgs base_args(void* ws, const Layout& L, const float* psf, const float* img
     a.eval_variant = L.eval_variant;
     a.os_ns = L.os_ns;
     a.conv_ty = L.conv_ty;
+    a.conv_rows = L.conv_rows;
     a.tot_wb = L.tot_wb;
     return a;
 }
@@ -1162,10 +1145,7 @@ gf_status ensure_bn_table(cudaStream_t s)
 // capture begins.
 gf_status prepare_conv(const Plan& pl)
 {
-    if (pl.method == GF_CONV_DIRECT) {
-        static int optin[64];
-        GF_CUDA(ensure_smem_optin_conv_direct(pl.st[0].P, optin));
-    }
+    if (pl.method == GF_CONV_DIRECT) GF_CUDA(ensure_smem_optin_conv_direct(pl.st[0].P, pl.L.conv_rows));
     return GF_OK;
 }
 
@@ -1376,8 +1356,6 @@ size_t gf_workspace_size_eval_batch(const gf_desc* d, const gf_batch* b)
 {
     if (!b || b->count < 1 || !b->H || !b->W) return 0;
     if (check_structure(d) != GF_OK) return 0;
-    const gf_desc db = batch_desc(d, b);
-    d = &db;
     for (int i = 0; i < b->count; ++i)
         if (check_stamp(d, b->H[i], b->W[i]) != GF_OK) return 0;
     if (check_fft(d, b->count, b->H, b->W) != GF_OK) return 0;
@@ -1392,8 +1370,6 @@ size_t gf_workspace_size_batch(const gf_desc* d, const gf_batch* b, const uint8_
 {
     if (!b || b->count < 1 || !b->H || !b->W) return 0;
     if (check_structure(d) != GF_OK) return 0;
-    const gf_desc db = batch_desc(d);
-    d = &db;
     for (int i = 0; i < b->count; ++i)
         if (check_stamp(d, b->H[i], b->W[i]) != GF_OK) return 0;
     Structure S;
@@ -1559,8 +1535,6 @@ static gf_status eval_batch_impl(const gf_desc* d, const gf_batch* b, const doub
     gf_status r = check_structure(d);
     if (r != GF_OK) return r;
     if (!b || b->count < 1 || !b->H || !b->W) return fail(GF_EINVAL, "bad batch");
-    const gf_desc db = batch_desc(d, b);
-    d = &db;
     for (int i = 0; i < b->count; ++i)
         if ((r = check_stamp(d, b->H[i], b->W[i])) != GF_OK) return r;
     if ((r = check_fft(d, b->count, b->H, b->W)) != GF_OK) return r;
@@ -1661,12 +1635,10 @@ static gf_status lm_fit_impl(const gf_desc* d, const gf_batch* b, double* params
                              const uint8_t* fixed, const double* lo, const double* hi,
                              const float* img, const float* sig, const float* psf,
                              const gf_lm_opts* opts, gf_lm_result* res, void* ws, size_t ws_bytes,
-                             gf_stream stream, bool batched)
+                             gf_stream stream)
 {
     gf_status r = check_structure(d);
     if (r != GF_OK) return r;
-    const gf_desc db = batched ? batch_desc(d) : *d;
-    d = &db;
     if (!b || b->count < 1 || !b->H || !b->W) return fail(GF_EINVAL, "bad batch");
     for (int i = 0; i < b->count; ++i)
         if ((r = check_stamp(d, b->H[i], b->W[i])) != GF_OK) return r;
@@ -1960,7 +1932,7 @@ gf_status gf_lm_fit_batch(const gf_desc* d, const gf_batch* b, double* params,
                           size_t ws_bytes, gf_stream stream)
 {
     return lm_fit_impl(d, b, params, fixed, nullptr, nullptr, img, sig, psf, opts, res, ws,
-                       ws_bytes, stream, true);
+                       ws_bytes, stream);
 }
 
 // The batch of a multi-start fit: stamp i repeated `starts` times (entry
@@ -2026,7 +1998,7 @@ gf_status gf_lm_fit_multistart(const gf_desc* d, const gf_batch* b, int starts,
     std::vector<double> p(starts_host, starts_host + (size_t)n * ns);
     std::vector<gf_lm_result> res((size_t)n);
     if ((r = lm_fit_impl(d, &m.b, p.data(), fixed, nullptr, nullptr, img, sig, psf, opts, res.data(),
-                         ws, ws_bytes, stream, true)) != GF_OK)
+                         ws, ws_bytes, stream)) != GF_OK)
         return r;
     // per stamp the fit with the lowest finite chi^2, the earliest start on ties
     for (int i = 0; i < b->count; ++i) {
@@ -2061,7 +2033,7 @@ gf_status gf_lm_fit(const gf_desc* d, double* params, const uint8_t* fixed, cons
     b.pix_off = &zero;
     b.psf_off = &zero;
     return lm_fit_impl(d, &b, params, fixed, lo, hi, img, sig, psf, opts, res, ws, ws_bytes,
-                       stream, false);
+                       stream);
 }
 
 }  // extern "C"

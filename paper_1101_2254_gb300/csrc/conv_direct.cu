@@ -10,7 +10,7 @@
 // device's tuning table (gf_autotune) or its defaults (TY 32, 8 CTAs per SM).  The
 // flipped PSF (rows padded with zeros to P4, a multiple of 4 taps) and the
 // (TY+P-1) x SW halo tile of the channel grid are staged in shared memory; for
-// PSFs up to 35 pixels the tile is double-buffered and filled by cp.async, so a
+// PSFs up to 35 pixels (39 with ROWS) the tile is double-buffered and filled by cp.async, so a
 // CTA's next tile arrives while its current one is summed.
 // A warp covers 16 x 32 outputs: lane 8 cg + rl owns the 8 contiguous columns
 // 8 cg .. 8 cg + 7 of rows rl and rl + 8.  For each tap row and group of 4
@@ -29,7 +29,16 @@
 // The outputs go back through shared memory (row stride TX + 1, conflict-free)
 // so that the global stores are coalesced rows.
 //
-// Each output accumulates its taps in the order v, then u, as a chain of FMAs.
+// Each output accumulates its taps in the order v, then u, as a chain of FMAs; with
+// ROWS each tap row is a chain of its own and the rows' sums are added in order.
+// ROWS is what the automatic method takes for P from 23 to 39 (capi.cu): the one
+// chain's round-off grows with its P^2 links, the rows' with P + P.  Each form in
+// float32 against 64 bits (restated in numpy, 64x64 galaxies of flux 1e5 to 1e7 on a
+// sky of 0.05), the worst pixel relative to itself / to the peak:
+//   P        one chain              tap rows               float32 FFT (96 or 128)
+//   23   2.8e-6 / 1.4e-6        4.1e-7 / 2.3e-7          4e-1 / 2.4e-7
+//   33   7.6e-6 / 2.8e-6        4.7e-7 / 2.3e-7          4e-1 / 2.1e-7
+//   39   9.6e-6 / 3.3e-6        5.5e-7 / 2.7e-7          2e-1 / 2.0e-7
 // The work is bound by the FP32 FMA pipe (2 P^2 flop per output pixel against
 // 8 bytes of HBM traffic), not by HBM.
 #include "gf_internal.cuh"
@@ -245,8 +254,9 @@ __device__ __forceinline__ void stage_tile_sync(float* es, const ConvItem& q, in
 // it's taps run, so the FMA pipe does not wait on global memory between items.
 // The generic kernel (larger PSFs, whose two tiles would not fit in shared
 // memory) stages each tile synchronously.  The sums are the same either way.
-template <int TX, int TY, int P4K>
-__global__ void __launch_bounds__(TX * TY / 16) k_conv_direct(PassArgs a)
+// (128 registers: 16 warps an SM, which is also what a 33 px PSF's tiles leave room for)
+template <int TX, int TY, int P4K, bool ROWS>
+__global__ void __launch_bounds__(TX * TY / 16, 512 / (TX * TY / 16)) k_conv_direct(PassArgs a)
 {
     pdl_entry();
     constexpr bool DB = P4K > 0;
@@ -331,8 +341,22 @@ __global__ void __launch_bounds__(TX * TY / 16) k_conv_direct(PassArgs a)
 #pragma unroll
             for (int o = 0; o < 8; ++o) acc[i][o] = 0.0f;
         if (active)
-            for (int v = 0; v < P; ++v)
-                tap_row<P4K>(acc, ks + v * P4, es + (r0 + v) * SW + c0, SW, P4, P - (P4 - 4));
+            for (int v = 0; v < P; ++v) {
+                if (!ROWS) {
+                    tap_row<P4K>(acc, ks + v * P4, es + (r0 + v) * SW + c0, SW, P4, P - (P4 - 4));
+                    continue;
+                }
+                float row[RPT][8];
+#pragma unroll
+                for (int i = 0; i < RPT; ++i)
+#pragma unroll
+                    for (int o = 0; o < 8; ++o) row[i][o] = 0.0f;
+                tap_row<P4K>(row, ks + v * P4, es + (r0 + v) * SW + c0, SW, P4, P - (P4 - 4));
+#pragma unroll
+                for (int i = 0; i < RPT; ++i)
+#pragma unroll
+                    for (int o = 0; o < 8; ++o) acc[i][o] += row[i][o];
+            }
 
         if (active && a.work && lane == 0) {
             const unsigned long long rows = (unsigned long long)min(16, q.H - q.ty0 - wr0);
@@ -408,7 +432,7 @@ constexpr int THIN_THREADS = 128;
 
 __host__ __device__ constexpr int thin_sw(int P4) { return 32 + P4; }
 
-template <int P>
+template <int P, bool ROWS>
 __global__ void __launch_bounds__(THIN_THREADS) k_conv_direct_thin(PassArgs a)
 {
     pdl_entry();
@@ -483,10 +507,17 @@ __global__ void __launch_bounds__(THIN_THREADS) k_conv_direct_thin(PassArgs a)
         for (int m = 0; m < P4 + 4; m += 4) *reinterpret_cast<float4*>(win + m) = *reinterpret_cast<const float4*>(er + m);
 #pragma unroll
         for (int m = 0; m < P4; m += 4) *reinterpret_cast<float4*>(k + m) = *reinterpret_cast<const float4*>(kr + m);
+        float row[4] = {0.0f, 0.0f, 0.0f, 0.0f};
 #pragma unroll
         for (int u = 0; u < P; ++u)
 #pragma unroll
-            for (int o = 0; o < 4; ++o) acc[o] = fmaf(k[u], win[u + o], acc[o]);
+            for (int o = 0; o < 4; ++o) {
+                float& x = ROWS ? row[o] : acc[o];
+                x = fmaf(k[u], win[u + o], x);
+            }
+        if (ROWS)
+#pragma unroll
+            for (int o = 0; o < 4; ++o) acc[o] += row[o];
     }
     const int rows = min(16, H - ty0), cols = min(32, W - tx0);
     if (a.work && tid == 0)
@@ -529,8 +560,6 @@ __global__ void __launch_bounds__(THIN_THREADS) k_conv_direct_thin(PassArgs a)
 
 }  // namespace
 
-cudaError_t ensure_smem_optin_conv_direct(int P, int* cache);
-
 // shared memory of k_conv_direct<TX, TY, P4K> for a P x P PSF: the taps and one
 // halo tile, or two where the kernel double-buffers (P4K > 0)
 template <int TX, int TY, int P4K>
@@ -541,53 +570,55 @@ size_t conv_smem(int P)
 }
 
 // one opt-in record per kernel instance and device
-template <int TX, int TY, int P4K>
+template <int TX, int TY, int P4K, bool ROWS>
 int* conv_optin_cache()
 {
     static int cache[64];
     return cache;
 }
 
-template <int TX, int TY, int P4K>
+template <int TX, int TY, int P4K, bool ROWS>
 cudaError_t launch_p4(const PassArgs& a, int kind, cudaStream_t s)
 {
-    GF_LAUNCH_PDL((k_conv_direct<TX, TY, P4K>), dim3(a.grid[kind]), dim3(TX * TY / 16),
+    GF_LAUNCH_PDL((k_conv_direct<TX, TY, P4K, ROWS>), dim3(a.grid[kind]), dim3(TX * TY / 16),
                   conv_smem<TX, TY, P4K>(a.P), s, a);
     GF_COUNT_LAUNCH();
     return cudaGetLastError();
 }
 
-template <int TX, int TY>
+// (tap rows are summed apart for P from 23 to 39 alone)
+template <int TX, int TY, bool ROWS>
 cudaError_t launch_tile_h(const PassArgs& a, int kind, cudaStream_t s)
 {
     switch ((a.P + 3) & ~3) {
-    case 4: return launch_p4<TX, TY, 4>(a, kind, s);
-    case 8: return launch_p4<TX, TY, 8>(a, kind, s);
-    case 12: return launch_p4<TX, TY, 12>(a, kind, s);
-    case 16: return launch_p4<TX, TY, 16>(a, kind, s);
-    case 20: return launch_p4<TX, TY, 20>(a, kind, s);
-    case 24: return launch_p4<TX, TY, 24>(a, kind, s);
-    case 28: return launch_p4<TX, TY, 28>(a, kind, s);
-    case 32: return launch_p4<TX, TY, 32>(a, kind, s);
-    case 36: return launch_p4<TX, TY, 36>(a, kind, s);
-    default: return launch_p4<TX, TY, 0>(a, kind, s);
+    case 4: return launch_p4<TX, TY, 4, false>(a, kind, s);
+    case 8: return launch_p4<TX, TY, 8, false>(a, kind, s);
+    case 12: return launch_p4<TX, TY, 12, false>(a, kind, s);
+    case 16: return launch_p4<TX, TY, 16, false>(a, kind, s);
+    case 20: return launch_p4<TX, TY, 20, false>(a, kind, s);
+    case 24: return launch_p4<TX, TY, 24, ROWS>(a, kind, s);
+    case 28: return launch_p4<TX, TY, 28, ROWS>(a, kind, s);
+    case 32: return launch_p4<TX, TY, 32, ROWS>(a, kind, s);
+    case 36: return launch_p4<TX, TY, 36, ROWS>(a, kind, s);
+    case 40: return launch_p4<TX, TY, ROWS ? 40 : 0, ROWS>(a, kind, s);
+    default: return launch_p4<TX, TY, 0, false>(a, kind, s);
     }
 }
 
-template <int TX>
+template <int TX, bool ROWS>
 cudaError_t launch_tile(const PassArgs& a, int kind, cudaStream_t s)
 {
     if (a.maxitems[kind] <= 0) return cudaSuccess;
-    return a.conv_ty == 16 ? launch_tile_h<TX, 16>(a, kind, s) : launch_tile_h<TX, 32>(a, kind, s);
+    return a.conv_ty == 16 ? launch_tile_h<TX, 16, ROWS>(a, kind, s) : launch_tile_h<TX, 32, ROWS>(a, kind, s);
 }
 
-template <int P>
+template <int P, bool ROWS>
 cudaError_t launch_thin(const PassArgs& a, cudaStream_t s)
 {
     constexpr int P4 = (P + 3) & ~3;
     constexpr size_t smem = sizeof(float) * (P * P4 + (16 + P - 1) * thin_sw(P4));
     static_assert(smem <= 48 * 1024, "no opt-in needed");
-    GF_LAUNCH_PDL(k_conv_direct_thin<P>, dim3((unsigned)(a.tot_wb * a.nchan)), dim3(THIN_THREADS), smem, s, a);
+    GF_LAUNCH_PDL((k_conv_direct_thin<P, ROWS>), dim3((unsigned)(a.tot_wb * a.nchan)), dim3(THIN_THREADS), smem, s, a);
     GF_COUNT_LAUNCH();
     return cudaGetLastError();
 }
@@ -602,32 +633,36 @@ cudaError_t launch_thin(const PassArgs& a, cudaStream_t s)
 // PSFs above 35 px keep the generic kernel, which also multiplies its padding taps.
 long long conv_thin_max_blocks(int P) { return P > 35 ? 0 : (P < 33 ? 4 : 3) * 152; }
 
+template <bool ROWS>
+cudaError_t launch_thin_p(const PassArgs& a, cudaStream_t s)
+{
+    switch (a.P) {
+    case 1: return launch_thin<1, false>(a, s);
+    case 3: return launch_thin<3, false>(a, s);
+    case 5: return launch_thin<5, false>(a, s);
+    case 7: return launch_thin<7, false>(a, s);
+    case 9: return launch_thin<9, false>(a, s);
+    case 11: return launch_thin<11, false>(a, s);
+    case 13: return launch_thin<13, false>(a, s);
+    case 15: return launch_thin<15, false>(a, s);
+    case 17: return launch_thin<17, false>(a, s);
+    case 19: return launch_thin<19, false>(a, s);
+    case 21: return launch_thin<21, false>(a, s);
+    case 23: return launch_thin<23, ROWS>(a, s);
+    case 25: return launch_thin<25, ROWS>(a, s);
+    case 27: return launch_thin<27, ROWS>(a, s);
+    case 29: return launch_thin<29, ROWS>(a, s);
+    case 31: return launch_thin<31, ROWS>(a, s);
+    case 33: return launch_thin<33, ROWS>(a, s);
+    case 35: return launch_thin<35, ROWS>(a, s);
+    default: return cudaErrorInvalidValue;
+    }
+}
+
 cudaError_t launch_conv_direct(const PassArgs& a, cudaStream_t s)
 {
-    const long long blocks = a.tot_wb * a.nchan;
-    if (blocks <= conv_thin_max_blocks(a.P)) {
-        switch (a.P) {
-        case 1: return launch_thin<1>(a, s);
-        case 3: return launch_thin<3>(a, s);
-        case 5: return launch_thin<5>(a, s);
-        case 7: return launch_thin<7>(a, s);
-        case 9: return launch_thin<9>(a, s);
-        case 11: return launch_thin<11>(a, s);
-        case 13: return launch_thin<13>(a, s);
-        case 15: return launch_thin<15>(a, s);
-        case 17: return launch_thin<17>(a, s);
-        case 19: return launch_thin<19>(a, s);
-        case 21: return launch_thin<21>(a, s);
-        case 23: return launch_thin<23>(a, s);
-        case 25: return launch_thin<25>(a, s);
-        case 27: return launch_thin<27>(a, s);
-        case 29: return launch_thin<29>(a, s);
-        case 31: return launch_thin<31>(a, s);
-        case 33: return launch_thin<33>(a, s);
-        case 35: return launch_thin<35>(a, s);
-        default: break;
-        }
-    }
+    if (a.tot_wb * a.nchan <= conv_thin_max_blocks(a.P))
+        return a.conv_rows ? launch_thin_p<true>(a, s) : launch_thin_p<false>(a, s);
     return launch_conv_direct_width(a, 0, s);
 }
 
@@ -635,44 +670,52 @@ cudaError_t launch_conv_direct(const PassArgs& a, cudaStream_t s)
 // tuner times its widths and shapes against each other
 cudaError_t launch_conv_direct_width(const PassArgs& a, int tile_w, cudaStream_t s)
 {
-    cudaError_t e = ensure_smem_optin_conv_direct(a.P, nullptr);
+    cudaError_t e = ensure_smem_optin_conv_direct(a.P, a.conv_rows);
     if (e != cudaSuccess) return e;
-    if (tile_w != 32 && (e = launch_tile<64>(a, WK_CONV, s)) != cudaSuccess) return e;
-    return tile_w != 64 ? launch_tile<32>(a, WK_CONV32, s) : cudaSuccess;
+    if (tile_w != 32) {
+        e = a.conv_rows ? launch_tile<64, true>(a, WK_CONV, s) : launch_tile<64, false>(a, WK_CONV, s);
+        if (e != cudaSuccess) return e;
+    }
+    if (tile_w == 64) return cudaSuccess;
+    return a.conv_rows ? launch_tile<32, true>(a, WK_CONV32, s) : launch_tile<32, false>(a, WK_CONV32, s);
 }
 
 // The shared-memory opt-in of the four tile shapes' kernels for a P x P PSF,
 // made before the first launch (and cached per device), so that a call made
 // before a stream capture leaves nothing to set inside it.
-template <int P4K>
+template <int P4K, bool ROWS>
 cudaError_t optin_p4(int P)
 {
-    cudaError_t e = ensure_smem_optin((const void*)k_conv_direct<64, 32, P4K>,
-                                      (int)conv_smem<64, 32, P4K>(P), conv_optin_cache<64, 32, P4K>());
+    cudaError_t e = ensure_smem_optin((const void*)k_conv_direct<64, 32, P4K, ROWS>,
+                                      (int)conv_smem<64, 32, P4K>(P), conv_optin_cache<64, 32, P4K, ROWS>());
     if (e == cudaSuccess)
-        e = ensure_smem_optin((const void*)k_conv_direct<32, 32, P4K>, (int)conv_smem<32, 32, P4K>(P),
-                              conv_optin_cache<32, 32, P4K>());
+        e = ensure_smem_optin((const void*)k_conv_direct<32, 32, P4K, ROWS>, (int)conv_smem<32, 32, P4K>(P),
+                              conv_optin_cache<32, 32, P4K, ROWS>());
     if (e == cudaSuccess)
-        e = ensure_smem_optin((const void*)k_conv_direct<64, 16, P4K>, (int)conv_smem<64, 16, P4K>(P),
-                              conv_optin_cache<64, 16, P4K>());
+        e = ensure_smem_optin((const void*)k_conv_direct<64, 16, P4K, ROWS>, (int)conv_smem<64, 16, P4K>(P),
+                              conv_optin_cache<64, 16, P4K, ROWS>());
     if (e == cudaSuccess)
-        e = ensure_smem_optin((const void*)k_conv_direct<32, 16, P4K>, (int)conv_smem<32, 16, P4K>(P),
-                              conv_optin_cache<32, 16, P4K>());
+        e = ensure_smem_optin((const void*)k_conv_direct<32, 16, P4K, ROWS>, (int)conv_smem<32, 16, P4K>(P),
+                              conv_optin_cache<32, 16, P4K, ROWS>());
     return e;
 }
 
-cudaError_t ensure_smem_optin_conv_direct(int P, int*)
+template <bool ROWS>
+cudaError_t optin_p(int P)
 {
     switch ((P + 3) & ~3) {
-    case 4: return optin_p4<4>(P);
-    case 8: return optin_p4<8>(P);
-    case 12: return optin_p4<12>(P);
-    case 16: return optin_p4<16>(P);
-    case 20: return optin_p4<20>(P);
-    case 24: return optin_p4<24>(P);
-    case 28: return optin_p4<28>(P);
-    case 32: return optin_p4<32>(P);
-    case 36: return optin_p4<36>(P);
-    default: return optin_p4<0>(P);
+    case 4: return optin_p4<4, false>(P);
+    case 8: return optin_p4<8, false>(P);
+    case 12: return optin_p4<12, false>(P);
+    case 16: return optin_p4<16, false>(P);
+    case 20: return optin_p4<20, false>(P);
+    case 24: return optin_p4<24, ROWS>(P);
+    case 28: return optin_p4<28, ROWS>(P);
+    case 32: return optin_p4<32, ROWS>(P);
+    case 36: return optin_p4<36, ROWS>(P);
+    case 40: return optin_p4<ROWS ? 40 : 0, ROWS>(P);
+    default: return optin_p4<0, false>(P);
     }
 }
+
+cudaError_t ensure_smem_optin_conv_direct(int P, int rows) { return rows ? optin_p<true>(P) : optin_p<false>(P); }

@@ -706,6 +706,7 @@ struct PassArgs {
     int eval_variant;          // 0 Sersic/disk/Gaussian, 1 with Moffat, 2 with King/Nuker/point
     int os_ns;                 // sub-samples per oversampled pixel (os_factor^2)
     int conv_ty;               // direct-convolution tile height (32 or 16)
+    int conv_rows;             // its tap rows are summed apart (the automatic method, P >= 23)
     int max_trial_slots;       // most trial-pass partial slots of one stamp (reduce blocks, or
                                // 16 x 32 output blocks with conv_chi2)
     int conv_chi2;             // an LM trial pass on the direct path or the one-CTA FFT: the
@@ -736,7 +737,7 @@ enum { PROF_MODEL = 0, PROF_CONV = 1, PROF_REDUCE = 2, PROF_LM = 3, PROF_CLASSES
 
 // per-device one-time opt-in to large dynamic shared memory for a kernel
 cudaError_t ensure_smem_optin(const void* func, int bytes, int* cache_per_device);
-cudaError_t ensure_smem_optin_conv_direct(int P, int* cache_per_device);
+cudaError_t ensure_smem_optin_conv_direct(int P, int rows);
 
 // ------------------------------------------------ programmatic dependent launch
 // The kernels of a pass are launched with programmatic stream serialization:
