@@ -88,7 +88,7 @@ __device__ __forceinline__ void fma_row_tail(float (&acc)[8], const float4 kk, c
 
 // One tap row v for the thread's RPT rows: er0 points at the first row's first
 // window column.  With the tap count P4K known at compile time (PSFs up to
-// 35 pixels) the loop over tap groups unrolls completely and the sliding
+// 35 pixels, 39 with ROWS) the loop over tap groups unrolls completely and the sliding
 // window costs no register moves; otherwise (P4K = 0) it runs over P4.
 template <int P4K>
 __device__ __forceinline__ void tap_row(float (&acc)[RPT][8], const float* kr, const float* er0,
@@ -249,7 +249,7 @@ __device__ __forceinline__ void stage_tile_sync(float* es, const ConvItem& q, in
 }
 
 // Work item = (channel, output tile of a listed stamp of this tile width).
-// With DB (the kernels specialised on the tap count, P <= 35) the halo tile is
+// With DB (the kernels specialised on the tap count, P <= 35, 39 with ROWS) the halo tile is
 // double-buffered: the cp.async copies of item it + 1 are in flight while item
 // it's taps run, so the FMA pipe does not wait on global memory between items.
 // The generic kernel (larger PSFs, whose two tiles would not fit in shared
@@ -342,20 +342,20 @@ __global__ void __launch_bounds__(TX * TY / 16, 512 / (TX * TY / 16)) k_conv_dir
             for (int o = 0; o < 8; ++o) acc[i][o] = 0.0f;
         if (active)
             for (int v = 0; v < P; ++v) {
-                if (!ROWS) {
+                if constexpr (ROWS) {
+                    float row[RPT][8];
+#pragma unroll
+                    for (int i = 0; i < RPT; ++i)
+#pragma unroll
+                        for (int o = 0; o < 8; ++o) row[i][o] = 0.0f;
+                    tap_row<P4K>(row, ks + v * P4, es + (r0 + v) * SW + c0, SW, P4, P - (P4 - 4));
+#pragma unroll
+                    for (int i = 0; i < RPT; ++i)
+#pragma unroll
+                        for (int o = 0; o < 8; ++o) acc[i][o] += row[i][o];
+                } else {
                     tap_row<P4K>(acc, ks + v * P4, es + (r0 + v) * SW + c0, SW, P4, P - (P4 - 4));
-                    continue;
                 }
-                float row[RPT][8];
-#pragma unroll
-                for (int i = 0; i < RPT; ++i)
-#pragma unroll
-                    for (int o = 0; o < 8; ++o) row[i][o] = 0.0f;
-                tap_row<P4K>(row, ks + v * P4, es + (r0 + v) * SW + c0, SW, P4, P - (P4 - 4));
-#pragma unroll
-                for (int i = 0; i < RPT; ++i)
-#pragma unroll
-                    for (int o = 0; o < 8; ++o) acc[i][o] += row[i][o];
             }
 
         if (active && a.work && lane == 0) {
@@ -515,9 +515,10 @@ __global__ void __launch_bounds__(THIN_THREADS) k_conv_direct_thin(PassArgs a)
                 float& x = ROWS ? row[o] : acc[o];
                 x = fmaf(k[u], win[u + o], x);
             }
-        if (ROWS)
+        if constexpr (ROWS) {
 #pragma unroll
             for (int o = 0; o < 4; ++o) acc[o] += row[o];
+        }
     }
     const int rows = min(16, H - ty0), cols = min(32, W - tx0);
     if (a.work && tid == 0)
