@@ -520,7 +520,6 @@ struct Plan {
     int method;            // GF_CONV_DIRECT, GF_CONV_FFT or GF_CONV_DFT_TC
     int Nx = 0, Ny = 0, cpc = 0;  // FFT geometry (method FFT)
     int small = 0;         // FFT: one CTA per transform (Nx, Ny in 32 x {3, 4, 5})
-    int toy = 0, tox = 0;  // small: outputs of a transform (the stamp's size)
     DftFactor fx, fy;      // DFT geometry (method DFT_TC)
 };
 
@@ -583,15 +582,7 @@ void plan_batch(const gf_desc* d, const Structure& S, int count, const int* H, c
         pl->Nx = fft_small_len(s0.We);
         pl->Ny = fft_small_len(s0.He);
         pl->small = pl->Nx > 0 && pl->Ny > 0;
-        pl->toy = s0.H;
-        pl->tox = s0.W;
     }
-    if (pl->small)  // the convolution's work items are the transform's tiles
-        for (int b = 0; b < count; ++b) {
-            const StampInfo& s = pl->st[b];
-            pc[b + 1] = pc[b] + ((s.H + pl->toy - 1) / pl->toy) * ((s.W + pl->tox - 1) / pl->tox);
-            pc32[b + 1] = 0;
-        }
     Layout& L = pl->L;
     memset(&L, 0, sizeof(L));
     L.max_red = max_red;
@@ -850,9 +841,6 @@ FFTArgs fft_args(void* ws, const Plan& pl)
     f.Ny = pl.Ny;
     f.cpc = pl.cpc;
     f.small = pl.small;
-    f.toy = pl.toy;
-    f.tox = pl.tox;
-    f.one_tile = pl.method == GF_CONV_FFT;
     f.px = make_fft_plan(pl.Nx);
     f.py = make_fft_plan(pl.Ny);
     f.tw_x = at<float2>(ws, pl.L.tw_x);

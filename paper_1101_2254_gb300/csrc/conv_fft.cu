@@ -29,7 +29,6 @@
 #include "fft.cuh"
 #include "gf_internal.cuh"
 #include "conv_fft.cuh"
-#include "reg_dft.cuh"
 #include "warp_fft.cuh"
 
 namespace {
@@ -325,541 +324,333 @@ __global__ void __launch_bounds__(WROW_WARPS * 32) k_fft_rows_inv_w(FFTArgs f, R
 }
 
 // ------------------------------------------- one CTA per transform (small grids)
-// For Nx = 8 MX and Ny = 8 MY with MX, MY in {12, 16, 20} (grids up to 160 x 160)
-// the whole convolution of one channel tile runs in one CTA: its half spectrum
+// For Nx = 32 MX and Ny = 32 MY with MX, MY in {3, 4, 5} (grids up to 160 x 160)
+// the whole convolution of one channel runs in one CTA: its half spectrum
 // (Ny x Kx complex values, at most 104 KB) stays in shared memory between the
 // three stages, so the only global traffic is the grid read, the PSF spectrum
 // read and the valid region written (in an LM trial pass, the image and sigma
 // read and the chi^2 partials of the 16 x 32 output blocks written instead of
-// the region).
-// The tile is the whole stamp where its grid fits (the FFT method), or
-// toy x tox outputs of a stamp of any size (the tiled method, overlap-save: the
-// tile's grid window is toy + P - 1 by tox + P - 1, at most Ny x Nx; toy and tox
-// are multiples of the 16 x 32 blocks of the trial partials).
-// The grid is persistent over the (tile, channel) items of the pass's work list,
-// channels innermost: the twiddle tables are built once per CTA, a stamp's PSF
-// spectrum is met by its channels one after the other, and stamps that have
-// left the LM loop cost nothing.
+// the region).  The CTAs walk the (stamp, channel) items of the pass's work list,
+// channels innermost: a stamp's PSF spectrum is met by its channels one after the
+// other, and stamps that have left the LM loop cost nothing.  Every transform is a
+// warp register FFT:
+//   rows     a warp per pair of grid rows, packed and unpacked as in the row
+//            kernels above;
+//   columns  a warp per spectrum column: forward FFT along y, product with the
+//            PSF spectrum, inverse FFT; the rows [row0, row0 + H) kept in place;
+//   rows     a warp per pair of output rows, inverse of the packing.
+// The PSF spectrum is made by the same kernel (PSF): the PSF, read wrapped,
+// through the row pass and the forward column FFT, stored per column in the
+// order the warp FFT leaves it in (lane l, register k2 holds bin
+// k2 + MY bitrev5(l)), so that the product reads it coalesced and needs no
+// reordering: hperm[k][MY l + k2] = Hhat[k2 + MY bitrev5(l)][k].
 //
-// What bounds it is instruction issue, so the transforms are split to need few:
-// a length-8M transform is an M-point DFT per residue n mod 8 (phase A) and an
-// 8-point DFT per k mod M (phase B), each in one thread's registers
-// (reg_dft.cuh), exchanged once through shared memory in place, with one
-// twiddle product between them:
-//   X[k2 + M k1] = sum_{n1 < 8} w_8^{n1 k1} w_N^{n1 k2} sum_{n2 < M} x[n1 + 8 n2] w_M^{n2 k2}
-// (the inverse runs B, then A).  About 19 operations a value and transform,
-// packed two to an instruction where they are additions.  The stages:
-//   rows     A on pairs of grid rows packed as one complex row, straight from
-//            global memory; B on the classes k2 and M - k2 together, whose
-//            outputs are each other's mirror images, so the two half spectra are
-//            unpacked in registers;
-//   columns  A; B, product with the PSF spectrum and the inverse B in one go; A;
-//   rows     the packing and B; A, whose outputs go to global memory (a trial
-//            pass brings them through shared memory, a warp per row pair).
-// A thread's row index and column advance so that the column phases touch
-// consecutive addresses; the row phases exchange through the pair's own two
-// spectrum rows at an odd stride (pair p of a group at p (Nx + 1), residue n1 at
-// 2 n1), free of bank conflicts.
-// The PSF spectrum is made by the same kernel (psf_mode): the PSF, read wrapped
-// and scaled, through the row phases and the forward column phases, stored as
-// hperm[k1][k2][kx] for ky = k2 + MY k1, the order in which phase B reads it.
-// Against the warp-shuffle transform (a warp per row pair or column, radix-2
-// stages by shuffles) that stood here: 21.7 against 40.8 thousand warp
-// instructions a transform, issued at 42 against 84 % (24 warps an SM and a
-// barrier a phase), so that alone it is not faster (Jacobian pass of 8,192 stamps
-// of 64x64, 57,344 transforms of 96x96: 2.16 ms then, 2.3 now); but as a
-// persistent kernel over the work list the passes of 8,192 fits' loop take 15.3 ms
-// for 17.0, and 512 fits of 48-256 px stamps 11.6 ms for 14.5.
-// threads: a group's phase B needs 16 MX of them.  Four CTAs of 192 (80 registers
-// each, 24 warps an SM) measured faster than four of 256 (64, spilling) and five
-// of 192 (64): 42.4, 43.8 and 47.1 ms on 8,192 fits of 64x64 stamps.
-constexpr int small_threads(int MX) { return 16 * MX; }
+// What bounds it is instruction issue.  Transforms in one thread's registers, with two
+// exchanges through shared memory, take half the instructions but a barrier a phase
+// at 24 warps an SM.  12 LM steps, us a step, these / those: one stamp of 64x64
+// 85 / 100, of 128x128 106 / 149, 16 of 128x128 152 / 202, 2,000 of 64x64 1,189 /
+// 1,271, 500 of 96x96 717 / 717, of 128x128 972 / 1,051.
+//
+// Warps a CTA: sixteen where shared memory holds one CTA an SM, 160 x 160 (with eight
+// the steps of 128x128 stamps above take 121, 168 and 1,115 us).
+constexpr int small_warps(int Nx, int Ny) { return Nx == 160 && Ny == 160 ? 16 : 8; }
+
+// Waves of CTAs a launch has at most.  One wave keeps its CTAs in step, all in the
+// same stage, and leaves SMs idle at its end; with a CTA for every stamp and channel, a
+// batch whose stamps have mostly left the loop launches thousands of them for
+// nothing.  8,192 fits of 64x64 stamps, convolution, ms, for one wave, four and a CTA
+// each: 15.9, 14.9, 17.2.
+constexpr int SMALL_WAVES = 4;
 
 struct SmallIO {
-    int toy, tox;         // outputs of a tile (a multiple of 16 x 32, or the stamp's H x W)
-    int one_tile;         // every stamp is one tile
-    const StampInfo* st;
-    const float* psf;     // psf_mode: the PSFs and their scale 1 / (4 Ny Nx)
-    float scale;
-    float2* hperm;        // per stamp Kx * Ny values (written in psf_mode)
-    int count;            // stamps (psf_mode)
-    int psf_mode;
-    float flops;          // a full tile's transform work (profiling)
+    const float* in;      // grids: problem p at in + p in_stride, rows x width, row stride ld
+    long long in_stride;  // (PSF: the PSFs, stamp b's at in + st[b].psf_off)
+    int ld, width, rows;
+    float* out;           // results: problem p at out + p out_stride, H x W
+    long long out_stride;
+    int row0, col0, H, W;
+    float2* hperm;        // per stamp Kx * Ny values (written with PSF)
+    int nchan;
+    const StampInfo* st;  // PSF: the stamps, how many, their PSFs' side,
+    int count, P, c;      // (P - 1) / 2
+    float scale;          // and 1 / (Ny Nx), which the PSFs are multiplied by
+    float flops;          // one transform's work (profiling)
 };
 
-// One (tile, channel) item as its CTA sees it, in shared memory: the phases read
-// what they need of it instead of carrying it in registers, and one thread
-// fills the next item's while the current one is transformed.
-struct TileItem {
-    const float* in;        // the grid window (or, in psf_mode, the PSF)
-    const float* img;       // the tile's image and sigma
-    const float* sig;
-    float* out;             // the tile's outputs
-    float2* hp;             // the stamp's PSF spectrum
-    long long slot;         // the tile's first trial partial
-    int W, We, c, P;        // the stamp's width, its grid's, (P - 1) / 2, P
-    int hO, wO;             // the tile's outputs
-    int rows, width;        // its grid window
-    int npair, ngrp, G;     // row pairs of the window, their exchange groups and a group's pairs
-    int ngo, Go;            // the same for the output rows
-    int ch;
-    int psf_mode;
-    float scale;            // psf_mode: the PSF's
-    float tmw, tmsky;       // a trial channel's weight and sky
-};
-
-// most row pairs of one exchange group: a thread per pair and class in phase B
-constexpr int SMALL_GROUP = 32;
-
-constexpr size_t small_smem(int MX, int MY)
+// the column transforms' register twiddles: the row set itself when Nx = Ny
+template <int MX, int MY>
+__device__ __forceinline__ const WarpTw<MY>& select_tw(const WarpTw<MX>& rx, const WarpTw<MY>& ry)
 {
-    // the half spectrum, the twiddle tables (rows of M + 1), the trial pass's
-    // row-pair sums per 32 columns
-    return sizeof(float2) * ((size_t)(8 * MY) * (4 * MX + 1) + 8 * (size_t)(MX + 1) + 8 * (size_t)(MY + 1) +
-                             (size_t)(4 * MY) * ((8 * MX) / 32)) + 2 * sizeof(TileItem);
+    if constexpr (MX == MY)
+        return rx;
+    else
+        return ry;
 }
 
-// CTAs per SM that the kernel's shared memory allows (227 KB per SM, 1 KB of
-// it taken by each CTA), at most four, which its register budget is held to
+// Shared memory, in float2: the twiddle table (tables, where Nx and Ny differ), whose
+// space a trial pass's row-pair chi^2 partials take, (Ny / 2) x (Nx / 32) CSum
+// values, once the lanes hold their twiddles; the half spectrum; one reordering row
+// per warp.
+constexpr size_t small_head(int Nx, int Ny)
+{
+    const size_t tables = (size_t)warp_fft_table_len(Nx) + (Nx == Ny ? 0 : (size_t)warp_fft_table_len(Ny));
+    const size_t part = (size_t)(Ny / 2) * (Nx / 32);
+    return tables > part ? tables : part;
+}
+
+constexpr size_t small_smem(int Nx, int Ny)
+{
+    return sizeof(float2) *
+           (small_head(Nx, Ny) + (size_t)Ny * (Nx / 2 + 1) + (size_t)small_warps(Nx, Ny) * (Nx > Ny ? Nx : Ny));
+}
+
+// CTAs per SM that this allows (228 KB per SM, 1 KB of it taken by each CTA: three
+// for 128 x 128 by a hair), at most four, which the register budget is held to.
+// (Five for 96 x 96 leave 48 registers, which spill: 12 LM steps of 2,000 stamps of
+// 64x64, 1,230 us a step for 1,198, a single stamp 94 for 90.)
 template <int MX, int MY>
 constexpr int small_ctas_per_sm()
 {
-    const int n = (int)((227u * 1024u) / (small_smem(MX, MY) + 1024));
+    const int n = (int)((228u * 1024u) / (small_smem(32 * MX, 32 * MY) + 1024));
     return n < 1 ? 1 : (n > 4 ? 4 : n);
 }
 
-// The phases of k_conv_fft_small, separated by barriers.
-template <int MX, int MY>
-struct TilePhases {
-    static constexpr int Nx = 8 * MX, Ny = 8 * MY, Kx = Nx / 2 + 1, NT = small_threads(MX);
-    static constexpr int HJ = MX / 2;  // class pairs of a row transform
-    static_assert(MX % 2 == 0 && MY % 2 == 0 && 2 * Kx > Nx && NT / HJ >= SMALL_GROUP,
-                  "the exchange fits the pair's rows, a group the block");
-
-    // slot of Y[n1][k2] in a pair's exchange area
-    static __device__ __forceinline__ int pos(int n1, int k2) { return (k2 >> 1) * 16 + 2 * n1 + (k2 & 1); }
-
-    // rows, phase A: pairs (y0, y0 + 1) of the grid window; rows >= rows are zeros
-    static __device__ __forceinline__ void rows_a(float2* spec, const float2* twx, const TileItem& I)
-    {
-#pragma unroll 1
-        for (int t = (int)threadIdx.x; t < 8 * I.npair; t += NT) {
-            const int pr = t >> 3, n1 = t & 7;
-            const int y0 = 2 * pr, y1 = y0 + 1;
-            float2 v[MX];
-            if (I.psf_mode) {  // psf[v][u] scale at ((v - c) mod Ny, (u - c) mod Nx)
-                const int P = I.P, c = I.c;
-                const float* in = I.in;
-                const int v0 = y0 <= c ? y0 + c : y0 + c - Ny, v1 = y1 <= c ? y1 + c : y1 + c - Ny;
-#pragma unroll
-                for (int n2 = 0; n2 < MX; ++n2) {
-                    const int x = n1 + 8 * n2, u = x <= c ? x + c : x + c - Nx;
-                    v[n2].x = u >= 0 && v0 >= 0 ? in[v0 * P + u] * I.scale : 0.0f;
-                    v[n2].y = u >= 0 && v1 >= 0 ? in[v1 * P + u] * I.scale : 0.0f;
-                }
-            } else {
-                const int We = I.We, width = I.width;
-                const float* r0 = I.in + (long long)y0 * We + n1;
-                const bool two = y1 < I.rows;
-#pragma unroll
-                for (int n2 = 0; n2 < MX; ++n2) {
-                    const bool cx = n1 + 8 * n2 < width;
-                    v[n2].x = cx ? r0[8 * n2] : 0.0f;
-                    v[n2].y = cx && two ? r0[We + 8 * n2] : 0.0f;
-                }
-            }
-            rdft<MX, false>(v);
-            const int G = I.G;
-            float2* e = spec + (pr / G) * (2 * G * Kx) + (pr % G) * (Nx + 1);
-            const float2* w = twx + n1 * (MX + 1);
-            e[pos(n1, 0)] = v[0];
-#pragma unroll
-            for (int k2 = 1; k2 < MX; ++k2) e[pos(n1, k2)] = c_mul(v[k2], w[k2]);
-        }
-    }
-
-    // rows, phase B and unpacking: with Z = A + i B (rows y0 and y1) the bins are
-    // A = Z[k] + conj Z[N-k], B = (Z[k] - conj Z[N-k]) / i, twice the spectra
-    // (the PSF's scale has the factor)
-    static __device__ __forceinline__ void rows_b(float2* spec, const TileItem& I)
-    {
-#pragma unroll 1
-        for (int g = 0; g < I.ngrp; ++g) {
-            const int G = I.G, np = min(G, I.npair - g * G);
-            const int t0 = (int)threadIdx.x, j = t0 / np, p = t0 - j * np;
-            const int jb = j == 0 ? HJ : MX - j;
-            float2 za[8], zb[8];
-            if (j < HJ) {
-                const float2* e = spec + g * (2 * G * Kx) + p * (Nx + 1);
-#pragma unroll
-                for (int n1 = 0; n1 < 8; ++n1) {
-                    za[n1] = e[pos(n1, j)];
-                    zb[n1] = e[pos(n1, jb)];
-                }
-            }
-            __syncthreads();
-            if (j < HJ) {
-                rdft8<false>(za);
-                rdft8<false>(zb);
-                float2* sa = spec + (g * G + p) * (2 * Kx);
-                auto unpack = [&](int k, float2 zk, float2 zm) {
-                    sa[k] = c2(zk.x + zm.x, zk.y - zm.y);
-                    sa[Kx + k] = c2(zk.y + zm.y, zm.x - zk.x);
-                };
-                // the mirror of (k1, j) is (7 - k1, MX - j), but the classes 0 and MX / 2
-                // mirror themselves
-#pragma unroll
-                for (int k1 = 0; k1 < 4; ++k1) {
-                    unpack(j + MX * k1, za[k1], j == 0 ? za[(8 - k1) % 8] : zb[7 - k1]);
-                    unpack(jb + MX * k1, zb[k1], j == 0 ? zb[7 - k1] : za[7 - k1]);
-                }
-                if (j == 0) unpack(4 * MX, za[4], za[4]);
-            }
-        }
-    }
-
-    // columns, phase A: value (n1 + 8 n2, k) sits at t + 8 Kx n2 for t = n1 Kx + k
-    static __device__ __forceinline__ void cols_a(float2* spec, const float2* twy, const TileItem& I)
-    {
-#pragma unroll 1
-        for (int t = (int)threadIdx.x; t < 8 * Kx; t += NT) {
-            const int n1 = t / Kx, hw = 2 * I.npair;
-            float2* col = spec + t;
-            float2 v[MY];
-#pragma unroll
-            for (int n2 = 0; n2 < MY; ++n2)
-                v[n2] = n1 + 8 * n2 < hw ? col[8 * Kx * n2] : c2(0.0f, 0.0f);
-            rdft<MY, false>(v);
-            const float2* w = twy + n1 * (MY + 1);
-            col[0] = v[0];
-#pragma unroll
-            for (int k2 = 1; k2 < MY; ++k2) col[8 * Kx * k2] = c_mul(v[k2], w[k2]);
-        }
-    }
-
-    // columns, phase B, the PSF product and the inverse's phase B
-    static __device__ __forceinline__ void cols_b(float2* spec, const TileItem& I)
-    {
-#pragma unroll 1
-        for (int t = (int)threadIdx.x; t < MY * Kx; t += NT) {
-            float2* col = spec + (t / Kx) * (8 * Kx) + t % Kx;
-            float2* hp = I.hp + t;
-            float2 v[8], h[8];
-            if (!I.psf_mode) {
-#pragma unroll
-                for (int k1 = 0; k1 < 8; ++k1) h[k1] = hp[k1 * (MY * Kx)];
-            }
-#pragma unroll
-            for (int n1 = 0; n1 < 8; ++n1) v[n1] = col[n1 * Kx];
-            rdft8<false>(v);
-            if (I.psf_mode) {
-#pragma unroll
-                for (int k1 = 0; k1 < 8; ++k1) hp[k1 * (MY * Kx)] = v[k1];
-                continue;
-            }
-#pragma unroll
-            for (int k1 = 0; k1 < 8; ++k1) v[k1] = c_mul(v[k1], h[k1]);
-            rdft8<true>(v);
-#pragma unroll
-            for (int n1 = 0; n1 < 8; ++n1) col[n1 * Kx] = v[n1];
-        }
-    }
-
-    // columns, the inverse's phase A; the rows [c, c + hO) are kept
-    static __device__ __forceinline__ void cols_ai(float2* spec, const float2* twy, const TileItem& I)
-    {
-#pragma unroll 1
-        for (int t = (int)threadIdx.x; t < 8 * Kx; t += NT) {
-            const int n1 = t / Kx, lo = I.c, hi = I.c + I.hO;
-            float2* col = spec + t;
-            const float2* w = twy + n1 * (MY + 1);
-            float2 v[MY];
-            v[0] = col[0];
-#pragma unroll
-            for (int k2 = 1; k2 < MY; ++k2) v[k2] = c_mulc(col[8 * Kx * k2], w[k2]);
-            rdft<MY, true>(v);
-#pragma unroll
-            for (int n2 = 0; n2 < MY; ++n2) {
-                const int y = n1 + 8 * n2;
-                if (y >= lo && y < hi) col[8 * Kx * n2] = v[n2];
-            }
-        }
-    }
-
-    // output rows of group g (np pairs): the packing Z = A + i B of rows (i0, i0 + 1)
-    // and the inverse's phase B
-    static __device__ __forceinline__ void out_b(float2* area, const TileItem& I, int g, int np)
-    {
-        const int t0 = (int)threadIdx.x, j = t0 / np, p = t0 - j * np;
-        const int jb = j == 0 ? HJ : MX - j;
-        float2 za[8], zb[8];
-        if (j < HJ) {
-            const float2* sa = area + p * (2 * Kx);
-            const bool has1 = 2 * (g * I.Go + p) + 1 < I.hO;
-            auto pack = [&](int k, float2& zk, float2& zm) {  // Z[k] and Z[N - k]
-                const float2 A = sa[k], B = has1 ? sa[Kx + k] : c2(0.0f, 0.0f);
-                zk = c2(A.x - B.y, A.y + B.x);
-                zm = c2(A.x + B.y, B.x - A.y);
-            };
-            // (k1, j) and its mirror, as in the unpacking
-            float2 ma[4], mb[4], mid = c2(0.0f, 0.0f), drop;
-#pragma unroll
-            for (int k1 = 0; k1 < 4; ++k1) {
-                pack(j + MX * k1, za[k1], ma[k1]);
-                pack(jb + MX * k1, zb[k1], mb[k1]);
-            }
-            if (j == 0) pack(4 * MX, mid, drop);
-#pragma unroll
-            for (int k1 = 0; k1 < 4; ++k1) {
-                za[7 - k1] = j != 0 ? mb[k1] : k1 < 3 ? ma[(k1 + 1) % 4] : mid;
-                zb[7 - k1] = j != 0 ? ma[k1] : mb[k1];
-            }
-            rdft8<true>(za);
-            rdft8<true>(zb);
-        }
-        __syncthreads();
-        if (j < HJ) {
-            float2* e = area + p * (Nx + 1);
-#pragma unroll
-            for (int n1 = 0; n1 < 8; ++n1) {
-                e[pos(n1, j)] = za[n1];
-                e[pos(n1, jb)] = zb[n1];
-            }
-        }
-        __syncthreads();
-    }
-
-    // and the inverse's phase A: the outputs to global memory, or (a trial pass) each
-    // pair's two rows of floats in place of its exchange area
-    static __device__ __forceinline__ void out_a(float2* area, const float2* twx, const TileItem& I, int g, int np, int trial)
-    {
-        // phase A: a thread per pair and residue
-#pragma unroll 1
-        for (int t = (int)threadIdx.x; t - (t & 31) < 8 * np; t += NT) {  // whole warps: a pair's eight threads share one
-            const int pa = t >> 3, n1 = t & 7;
-            float2* e = area + pa * (Nx + 1);
-            float2 v[MX];
-            if (pa < np) {
-                const float2* w = twx + n1 * (MX + 1);
-                v[0] = e[pos(n1, 0)];
-#pragma unroll
-                for (int k2 = 1; k2 < MX; ++k2) v[k2] = c_mulc(e[pos(n1, k2)], w[k2]);
-                rdft<MX, true>(v);
-            }
-            if (!trial) {
-                if (pa < np) {
-                    const int i0 = 2 * (g * I.Go + pa), c = I.c, W = I.W, wO = I.wO;
-                    float* o0 = I.out + (long long)i0 * W + n1 - c;
-                    const bool has1 = i0 + 1 < I.hO;
-#pragma unroll
-                    for (int n2 = 0; n2 < MX; ++n2) {
-                        const int jx = n1 + 8 * n2 - c;
-                        if (jx >= 0 && jx < wO) {
-                            o0[8 * n2] = v[n2].x;
-                            if (has1) o0[W + 8 * n2] = v[n2].y;
-                        }
-                    }
-                }
-                continue;
-            }
-            __syncwarp();  // the pair's exchange area becomes its two rows of floats
-            if (pa < np) {
-                float* rowsf = reinterpret_cast<float*>(e);
-#pragma unroll
-                for (int n2 = 0; n2 < MX; ++n2) {
-                    rowsf[n1 + 8 * n2] = v[n2].x;
-                    rowsf[Nx + n1 + 8 * n2] = v[n2].y;
-                }
-            }
-        }
-    }
-
-    // a trial pass: each row pair's chi^2 per 32 columns
-    static __device__ __forceinline__ void out_chi2(const float2* area, CSum* part, const TileItem& I, int g, int np)
-    {
-        const int warp = threadIdx.x >> 5, l = threadIdx.x & 31;
-        const int hO = I.hO, wO = I.wO, W = I.W, c = I.c, nbx = (wO + 31) / 32;
-        const float tmw = I.tmw, tmsky = I.tmsky;
-        const float* img = I.img;
-        const float* sig = I.sig;
-#pragma unroll 1
-        for (int q = warp; q < np; q += NT / 32) {
-            const float* rowsf = reinterpret_cast<const float*>(area + q * (Nx + 1)) + c;
-            const int r0 = 2 * (g * I.Go + q);
-#pragma unroll 1
-            for (int t = 0; t < nbx; ++t) {
-                const int jx = l + 32 * t;
-                CSum cs = {0.0f, 0.0f};
-                if (jx < wO) {
-#pragma unroll
-                    for (int r = 0; r < 2; ++r) {
-                        if (r == 1 && r0 + 1 >= hO) break;
-                        const long long px = (long long)(r0 + r) * W + jx;
-                        const float d = __ldg(&img[px]), sg = __ldg(&sig[px]);
-                        if (isfinite(d) && isfinite(sg) && sg > 0.0f) {
-                            const float m = rowsf[r * Nx + jx];
-                            const float zr = (d - fmaf(tmw, m, tmsky)) / sg;
-                            csum_add(cs, zr * zr);
-                        }
-                    }
-                }
-#pragma unroll
-                for (int o = 16; o > 0; o >>= 1) {
-                    CSum other;
-                    other.s = __shfl_down_sync(0xffffffffu, cs.s, o);
-                    other.c = __shfl_down_sync(0xffffffffu, cs.c, o);
-                    cs = csum_merge(cs, other);
-                }
-                if (l == 0) part[(g * I.Go + q) * nbx + t] = cs;
-            }
-        }
-    }
-};
-
-template <int MX, int MY>
-__global__ void __launch_bounds__(small_threads(MX), small_ctas_per_sm<MX, MY>()) k_conv_fft_small(
+template <int MX, int MY, bool PSF>
+__global__ void __launch_bounds__(32 * small_warps(32 * MX, 32 * MY), small_ctas_per_sm<MX, MY>()) k_conv_fft_small(
     const __grid_constant__ SmallIO io, const __grid_constant__ PassArgs a, const float2* tw_x, const float2* tw_y)
 {
     pdl_entry();
-    constexpr int Nx = 8 * MX, Ny = 8 * MY, Kx = Nx / 2 + 1, NT = small_threads(MX);
-    constexpr int HJ = MX / 2;    // class pairs of a row transform
-    using Ph = TilePhases<MX, MY>;
-    static_assert(sizeof(CSum) == sizeof(float2), "a partial takes one float2 slot");
+    constexpr int Nx = 32 * MX, Ny = 32 * MY, Kx = Nx / 2 + 1;
+    constexpr int NZ = Nx > Ny ? Nx : Ny, NW = small_warps(Nx, Ny);
     extern __shared__ __align__(16) float2 sm[];
-    float2* spec = sm;                    // Ny rows of stride Kx (odd)
-    float2* twx = spec + Ny * Kx;         // w_Nx^{n1 k2} at n1 (MX + 1) + k2
-    float2* twy = twx + 8 * (MX + 1);     // w_Ny^{n1 k2} at n1 (MY + 1) + k2
-    CSum* part = reinterpret_cast<CSum*>(twy + 8 * (MY + 1));
-    TileItem* info = reinterpret_cast<TileItem*>(part + 4 * MY * (Nx / 32));
-    const int tid = threadIdx.x;
-    for (int t = tid; t < 8 * MX; t += NT) twx[(t / MX) * (MX + 1) + t % MX] = tw_x[(t / MX) * (t % MX)];
-    for (int t = tid; t < 8 * MY; t += NT) twy[(t / MY) * (MY + 1) + t % MY] = tw_y[(t / MY) * (t % MY)];
-    const int nchan = io.psf_mode ? 1 : a.nchan;
-    const int n = io.psf_mode ? io.count : *a.wl.n;
-    const int* pre = io.psf_mode ? nullptr : a.wl.pre + WK_CONV * (a.count + 1);
-    const long long items = (long long)(io.one_tile ? n : pre[n]) * nchan;
-    // this CTA's share, spread evenly
-    const long long it0 = items * blockIdx.x / gridDim.x, it1 = items * (blockIdx.x + 1) / gridDim.x;
-    int hint = -1;
-    auto fill = [&](long long it, TileItem& q) {
-        const int tile = (int)(it / nchan), ch = (int)(it - (long long)tile * nchan);
-        const int li = io.one_tile ? tile : wl_locate(pre, n, tile, hint);
-        const int b = io.psf_mode ? tile : a.wl.ids[li];
-        const StampInfo& st = io.st[b];
-        int ty0 = 0, tx0 = 0;
-        if (!io.one_tile) {
-            const int t = tile - pre[li], tiles_x = (st.W + io.tox - 1) / io.tox;
-            ty0 = (t / tiles_x) * io.toy;
-            tx0 = (t % tiles_x) * io.tox;
+    const int items = (PSF ? io.count : *a.wl.n) * io.nchan;
+    if ((int)blockIdx.x >= items) return;  // whole CTA
+    float2* twx = sm;
+    float2* twy = twx + (Nx == Ny ? 0 : warp_fft_table_len(Nx));
+    float2* spec = sm + small_head(Nx, Ny);  // Ny x Kx (row stride Kx: odd)
+    const int warp = threadIdx.x >> 5, l = threadIdx.x & 31;
+    float2* z = spec + Ny * Kx + warp * NZ;       // the warp's reordering buffer
+    for (int t = threadIdx.x; t < Nx; t += blockDim.x) twx[warp_fft_pad(t)] = tw_x[t];
+    if (Nx != Ny)
+        for (int t = threadIdx.x; t < Ny; t += blockDim.x) twy[warp_fft_pad(t)] = tw_y[t];
+    __syncthreads();
+    // the lane's twiddles for every transform of the CTA (one set when Nx = Ny)
+    WarpTw<MX> rx;
+    warp_tw_load<MX>(rx, twx);
+    WarpTw<MY> ry_own;
+    if constexpr (MX != MY) warp_tw_load<MY>(ry_own, twy);
+    const WarpTw<MY>& ry = select_tw<MX, MY>(rx, ry_own);
+    const int br = bitrev5(l);
+#pragma unroll 1
+    for (int it = blockIdx.x; it < items; it += gridDim.x) {
+        __syncthreads();  // the previous item is done with the spectrum
+        const int li = it / io.nchan, ch = it - li * io.nchan;
+        const int b = PSF ? li : a.wl.ids[li];
+        const long long p = (long long)b * io.nchan + ch;
+        // rows: pairs (y0, y0 + 1) of the grid; rows >= rows are zeros
+        const int npair = (io.rows + 1) / 2, hw = 2 * npair;  // spectrum rows written
+        const float* in = io.in + (PSF ? (long long)io.st[b].psf_off : p * io.in_stride);
+        // the warp's next row pair is loaded while the current one is transformed
+        auto load_pair = [&](int pr, float2 (&w)[MX]) {
+            const int y0 = 2 * pr, y1 = y0 + 1;
+            if constexpr (PSF) {  // psf[v][u] scale at ((v - c) mod Ny, (u - c) mod Nx)
+                const int v0 = y0 <= io.c ? y0 + io.c : y0 + io.c - Ny, v1 = y1 <= io.c ? y1 + io.c : y1 + io.c - Ny;
+#pragma unroll
+                for (int j = 0; j < MX; ++j) {
+                    const int x = l + 32 * j, u = x <= io.c ? x + io.c : x + io.c - Nx;
+                    w[j].x = u >= 0 && v0 >= 0 ? in[v0 * io.P + u] * io.scale : 0.0f;
+                    w[j].y = u >= 0 && v1 >= 0 ? in[v1 * io.P + u] * io.scale : 0.0f;
+                }
+            } else {
+#pragma unroll
+                for (int j = 0; j < MX; ++j) {
+                    const int x = l + 32 * j;
+                    const bool cx = x < io.width;
+                    const float va = cx ? in[(long long)y0 * io.ld + x] : 0.0f;
+                    const float vb = (cx && y1 < io.rows) ? in[(long long)y1 * io.ld + x] : 0.0f;
+                    w[j] = make_float2(va, vb);
+                }
+            }
+        };
+        float2 vn[MX];
+        if (warp < npair) load_pair(warp, vn);
+        for (int pr = warp; pr < npair; pr += NW) {
+            const int y0 = 2 * pr, y1 = y0 + 1;
+            float2 v[MX];
+#pragma unroll
+            for (int j = 0; j < MX; ++j) v[j] = vn[j];
+            if (pr + NW < npair) load_pair(pr + NW, vn);
+            warp_fft_r<MX, false>(v, rx);
+#pragma unroll
+            for (int k2 = 0; k2 < MX; ++k2) z[k2 + MX * br] = v[k2];
+            __syncwarp();
+            for (int k = l; k < Kx; k += 32) {
+                const float2 zk = z[k], zm = cconj(z[(Nx - k) % Nx]);
+                const float2 s = cadd(zk, zm), d = csub(zk, zm);
+                // A = (Z[k] + conj Z[N-k]) / 2,  B = (Z[k] - conj Z[N-k]) / (2i)
+                spec[y0 * Kx + k] = make_float2(0.5f * s.x, 0.5f * s.y);
+                spec[y1 * Kx + k] = make_float2(0.5f * d.y, -0.5f * d.x);
+            }
+            __syncwarp();
         }
-        q.W = st.W;
-        q.We = st.We;
-        q.c = st.c;
-        q.P = st.P;
-        q.ch = ch;
-        q.psf_mode = io.psf_mode;
-        q.scale = io.scale;
-        q.hp = io.hperm + (long long)b * Kx * Ny;
-        if (io.psf_mode) {
-            q.in = io.psf + st.psf_off;
-            q.hO = q.wO = 0;
-            q.rows = Ny;
-            q.width = Nx;
-        } else {
-            const long long at = (long long)ty0 * st.W + tx0;
-            q.in = a.ext + ext_index(st, nchan, ch) + (long long)ty0 * st.We + tx0;
-            q.out = a.y + y_index(st, nchan, ch) + at;
-            q.hO = min(io.toy, st.H - ty0);
-            q.wO = min(io.tox, st.W - tx0);
-            q.rows = q.hO + 2 * st.c;
-            q.width = q.wO + 2 * st.c;
+        __syncthreads();
+        // columns
+        float2* hp = io.hperm + (long long)b * Kx * Ny;
+        for (int k = warp; k < Kx; k += NW) {
+            float2* hk = hp + (long long)k * Ny + MY * l;
+            float2 h[MY];  // the PSF spectrum's column, loaded before the transform
+            if constexpr (!PSF) {
+#pragma unroll
+                for (int k2 = 0; k2 < MY; ++k2) h[k2] = hk[k2];
+            }
+            float2 v[MY];
+#pragma unroll
+            for (int j = 0; j < MY; ++j) {
+                const int y = l + 32 * j;
+                v[j] = y < hw ? spec[y * Kx + k] : make_float2(0.0f, 0.0f);
+            }
+            warp_fft_r<MY, false>(v, ry);
+            if constexpr (PSF) {
+#pragma unroll
+                for (int k2 = 0; k2 < MY; ++k2) hk[k2] = v[k2];
+            } else {
+#pragma unroll
+                for (int k2 = 0; k2 < MY; ++k2) z[k2 + MY * br] = cmul(v[k2], h[k2]);
+                __syncwarp();
+#pragma unroll
+                for (int j = 0; j < MY; ++j) v[j] = z[l + 32 * j];
+                __syncwarp();
+                warp_fft_r<MY, true>(v, ry);
+#pragma unroll
+                for (int k2 = 0; k2 < MY; ++k2) {
+                    const int y = k2 + MY * br;
+                    if (y >= io.row0 && y < io.row0 + io.H) spec[y * Kx + k] = v[k2];
+                }
+            }
+        }
+        if constexpr (!PSF) {
+            __syncthreads();
+            // rows: inverse of the packing, output rows (i0, i0 + 1).  In an LM trial
+            // pass (a.conv_chi2) nothing is written: each row pair's chi^2 per 32
+            // columns goes to part[pair][column block] (the twiddle tables' space), and
+            // the 16 x 32 blocks' sums to the stamp's partial slots.
+            float* out = io.out + p * io.out_stride;
+            static_assert(sizeof(CSum) == sizeof(float2), "a partial takes one float2 slot");
+            CSum* part = reinterpret_cast<CSum*>(sm);
+            const int nbx = (io.W + 31) / 32;
+            const float* img = nullptr;
+            const float* sig = nullptr;
+            float tmw = 0.0f, tmsky = 0.0f;
             if (a.conv_chi2) {
+                const StampInfo& st = a.st[b];
                 const Channel& chn = a.chan[(long long)b * a.chan_stride + ch];
-                q.tmw = chn.mweight;
-                q.tmsky = chn.msky;
-                q.img = a.img + st.pix_off + at;
-                q.sig = a.sig + st.pix_off + at;
-                q.slot = st.wb_off + (long long)(ty0 / 16) * ((st.W + 31) / 32) + tx0 / 32;
+                tmw = chn.mweight;
+                tmsky = chn.msky;
+                img = a.img + st.pix_off;
+                sig = a.sig + st.pix_off;
             }
-        }
-        // row pairs come in groups of G (the last one may be smaller), each
-        // exchanging through its own rows
-        q.npair = (q.rows + 1) / 2;
-        q.ngrp = (q.npair + SMALL_GROUP - 1) / SMALL_GROUP;
-        q.G = (q.npair + q.ngrp - 1) / q.ngrp;
-        const int npo = (q.hO + 1) / 2;
-        q.ngo = (npo + SMALL_GROUP - 1) / SMALL_GROUP;
-        q.Go = q.ngo ? (npo + q.ngo - 1) / q.ngo : 0;
-    };
-    if (it0 < it1 && tid == NT - 1) fill(it0, info[0]);
-    for (long long it = it0; it < it1; ++it) {
-        __syncthreads();  // the previous item is done with the spectrum, this one's info is there
-        const TileItem& I = info[(it - it0) & 1];
-        if (it + 1 < it1 && tid == NT - 1) fill(it + 1, info[(it + 1 - it0) & 1]);
-        Ph::rows_a(spec, twx, I);
-        __syncthreads();
-        Ph::rows_b(spec, I);
-        __syncthreads();
-        Ph::cols_a(spec, twy, I);
-        __syncthreads();
-        Ph::cols_b(spec, I);
-        if (io.psf_mode) continue;
-        __syncthreads();
-        Ph::cols_ai(spec, twy, I);
-        __syncthreads();
-        // output rows.  In an LM trial pass (a.conv_chi2) nothing is written: each
-        // row pair's chi^2 per 32 columns goes to part[pair][column block], and the
-        // 16 x 32 blocks' sums to the stamp's partial slots.
-        for (int g = 0; g < I.ngo; ++g) {
-            const int np = min(I.Go, (I.hO + 1) / 2 - g * I.Go);
-            float2* area = spec + (I.c + 2 * g * I.Go) * Kx;
-            Ph::out_b(area, I, g, np);
-            __syncthreads();
-            Ph::out_a(area, twx, I, g, np, a.conv_chi2);
-            if (!a.conv_chi2) continue;
-            __syncthreads();
-            Ph::out_chi2(area, part, I, g, np);
-        }
-        if (a.conv_chi2) {
-            // each 16 x 32 block: its 8 row pairs' partials merged in row order
-            __syncthreads();
-            const int nby = (I.hO + 15) / 16, nbw = (I.W + 31) / 32, nbx = (I.wO + 31) / 32, npo = (I.hO + 1) / 2;
-            for (int q = tid; q < nby * nbx; q += NT) {
-                const int by = q / nbx, bx = q - by * nbx;
-                CSum cs = part[(8 * by) * nbx + bx];
-                for (int pr = 8 * by + 1; pr < min(npo, 8 * by + 8); ++pr)
-                    cs = csum_merge(cs, part[pr * nbx + bx]);
-                a.partial[(I.slot + (long long)by * nbw + bx) * nchan + I.ch] = cs.s + cs.c;
+            for (int pr = warp; 2 * pr < io.H; pr += NW) {
+                const int i0 = 2 * pr, i1 = i0 + 1;
+                const bool has1 = i1 < io.H;
+                const float2* sa = spec + (io.row0 + i0) * Kx;
+                const float2* sb = spec + (io.row0 + (has1 ? i1 : i0)) * Kx;
+                float2 v[MX];
+#pragma unroll
+                for (int j = 0; j < MX; ++j) {
+                    const int k = l + 32 * j;
+                    float2 A, Bv;
+                    if (k < Kx) {
+                        A = sa[k];
+                        Bv = sb[k];
+                    } else {
+                        A = cconj(sa[Nx - k]);
+                        Bv = cconj(sb[Nx - k]);
+                    }
+                    if (!has1) Bv = make_float2(0.0f, 0.0f);
+                    v[j] = make_float2(A.x - Bv.y, A.y + Bv.x);  // A + i B
+                }
+                warp_fft_r<MX, true>(v, rx);
+#pragma unroll
+                for (int k2 = 0; k2 < MX; ++k2) z[k2 + MX * br] = v[k2];
+                __syncwarp();
+                if (a.conv_chi2) {
+                    for (int t = 0; t < nbx; ++t) {
+                        const int j = l + 32 * t;
+                        CSum cs = {0.0f, 0.0f};
+                        if (j < io.W) {
+                            const float2 w = z[io.col0 + j];
+#pragma unroll
+                            for (int r = 0; r < 2; ++r) {
+                                if (r == 1 && !has1) break;
+                                const long long px = (long long)(i0 + r) * io.W + j;
+                                const float d = __ldg(&img[px]), sg = __ldg(&sig[px]);
+                                if (isfinite(d) && isfinite(sg) && sg > 0.0f) {
+                                    const float zr = (d - fmaf(tmw, r ? w.y : w.x, tmsky)) / sg;
+                                    csum_add(cs, zr * zr);
+                                }
+                            }
+                        }
+#pragma unroll
+                        for (int o = 16; o > 0; o >>= 1) {
+                            CSum other;
+                            other.s = __shfl_down_sync(0xffffffffu, cs.s, o);
+                            other.c = __shfl_down_sync(0xffffffffu, cs.c, o);
+                            cs = csum_merge(cs, other);
+                        }
+                        if (l == 0) part[pr * nbx + t] = cs;
+                    }
+                } else {
+                    for (int j = l; j < io.W; j += 32) {
+                        const float2 w = z[io.col0 + j];
+                        out[(long long)i0 * io.W + j] = w.x;
+                        if (has1) out[(long long)i1 * io.W + j] = w.y;
+                    }
+                }
+                __syncwarp();
             }
+            if (a.conv_chi2) {
+                // each 16 x 32 block: its 8 row pairs' partials merged in row order
+                __syncthreads();
+                const int npo = (io.H + 1) / 2, nby = (io.H + 15) / 16;
+                const StampInfo& st = a.st[b];
+                for (int q = threadIdx.x; q < nby * nbx; q += blockDim.x) {
+                    const int by = q / nbx, bx = q - by * nbx;
+                    CSum cs = part[(8 * by) * nbx + bx];
+                    for (int pr = 8 * by + 1; pr < min(npo, 8 * by + 8); ++pr)
+                        cs = csum_merge(cs, part[pr * nbx + bx]);
+                    a.partial[((long long)st.wb_off + q) * io.nchan + ch] = cs.s + cs.c;
+                }
+            }
+            if (a.work && threadIdx.x == 0) atomicAdd(&a.work[PROF_CONV], (unsigned long long)io.flops);
         }
-        if (a.work && tid == 0) atomicAdd(&a.work[PROF_CONV], (unsigned long long)io.flops);
     }
 }
 
-template <int MX, int MY>
+template <int MX, int MY, bool PSF>
 cudaError_t launch_small_t(const SmallIO& io, const PassArgs& a, const FFTArgs& f, long long items,
                            cudaStream_t s)
 {
     static int optin[64];
-    const size_t smem = small_smem(MX, MY);
-    cudaError_t e = ensure_smem_optin((const void*)k_conv_fft_small<MX, MY>, (int)smem, optin);
+    const size_t smem = small_smem(32 * MX, 32 * MY);
+    cudaError_t e = ensure_smem_optin((const void*)k_conv_fft_small<MX, MY, PSF>, (int)smem, optin);
     if (e != cudaSuccess) return e;
-    const int grid = (int)std::min<long long>(items, 152LL * small_ctas_per_sm<MX, MY>());
-    GF_LAUNCH_PDL(k_conv_fft_small<MX, MY>, dim3(grid), dim3(small_threads(MX)), smem, s, io, a,
+    const int grid = (int)std::min<long long>(items, SMALL_WAVES * 152LL * small_ctas_per_sm<MX, MY>());
+    GF_LAUNCH_PDL((k_conv_fft_small<MX, MY, PSF>), dim3(grid), dim3(32 * small_warps(32 * MX, 32 * MY)), smem, s, io, a,
                   (const float2*)f.tw_x, (const float2*)f.tw_y);
     GF_COUNT_LAUNCH();
     return cudaSuccess;
 }
 
+template <bool PSF>
 cudaError_t launch_small(const SmallIO& io, const PassArgs& a, const FFTArgs& f, long long items,
                          cudaStream_t s)
 {
-    switch (f.Nx * 256 + f.Ny) {
-#define SMALL_CASE(NX_, NY_) \
-    case NX_ * 256 + NY_: return launch_small_t<NX_ / 8, NY_ / 8>(io, a, f, items, s);
-        SMALL_CASE(96, 96) SMALL_CASE(96, 128) SMALL_CASE(96, 160)
-        SMALL_CASE(128, 96) SMALL_CASE(128, 128) SMALL_CASE(128, 160)
-        SMALL_CASE(160, 96) SMALL_CASE(160, 128) SMALL_CASE(160, 160)
+    switch ((f.Nx / 32) * 8 + f.Ny / 32) {
+#define SMALL_CASE(MX_, MY_) \
+    case MX_ * 8 + MY_: return launch_small_t<MX_, MY_, PSF>(io, a, f, items, s);
+        SMALL_CASE(3, 3) SMALL_CASE(3, 4) SMALL_CASE(3, 5)
+        SMALL_CASE(4, 3) SMALL_CASE(4, 4) SMALL_CASE(4, 5)
+        SMALL_CASE(5, 3) SMALL_CASE(5, 4) SMALL_CASE(5, 5)
 #undef SMALL_CASE
     default: return cudaErrorInvalidValue;
     }
@@ -1010,14 +801,17 @@ cudaError_t launch_fft_psf(const FFTArgs& f, int count, const StampInfo* st, con
     if (f.small) {
         SmallIO io;
         memset(&io, 0, sizeof(io));
-        io.one_tile = 1;
-        io.st = st;
-        io.psf = psf;
-        io.scale = (float)(0.25 / ((double)f.Ny * (double)f.Nx));  // (see the unpacking)
+        io.in = psf;
+        io.width = f.Nx;
+        io.rows = f.Ny;
         io.hperm = f.hhat;
+        io.nchan = 1;
+        io.st = st;
         io.count = count;
-        io.psf_mode = 1;
-        const cudaError_t e = launch_small(io, none, f, count, s);
+        io.P = f.st0.P;
+        io.c = f.st0.c;
+        io.scale = (float)(1.0 / ((double)f.Ny * (double)f.Nx));
+        const cudaError_t e = launch_small<true>(io, none, f, count, s);
         return e != cudaSuccess ? e : cudaGetLastError();
     }
     cudaError_t e = optin_all(f);
@@ -1057,21 +851,28 @@ cudaError_t launch_conv_fft(const PassArgs& a, const FFTArgs& f, float2* spec, c
 {
     const StampInfo& s0 = f.st0;  // uniform stamp geometry (host copy)
     const int Kx = f.Nx / 2 + 1;
+    const int nprob = a.count * a.nchan;
     if (f.small) {
         SmallIO io;
         memset(&io, 0, sizeof(io));
-        io.toy = f.toy;
-        io.tox = f.tox;
-        io.one_tile = f.one_tile;
-        io.st = a.st;
+        io.in = a.ext;
+        io.in_stride = (long long)s0.He * s0.We;
+        io.ld = s0.We;
+        io.width = s0.We;
+        io.rows = s0.He;
+        io.out = a.y;
+        io.out_stride = (long long)s0.H * s0.W;
+        io.row0 = s0.c;
+        io.col0 = s0.c;
+        io.H = s0.H;
+        io.W = s0.W;
         io.hperm = f.hhat;
-        const int He = f.toy + 2 * s0.c;
-        io.flops = (float)(((He + 1) / 2 + (f.toy + 1) / 2) * 5.0 * f.Nx * log2((double)f.Nx) +
+        io.nchan = a.nchan;
+        io.flops = (float)(((s0.He + 1) / 2 + (s0.H + 1) / 2) * 5.0 * f.Nx * log2((double)f.Nx) +
                            Kx * (10.0 * f.Ny * log2((double)f.Ny) + 6.0 * f.Ny));
-        const cudaError_t e = launch_small(io, a, f, a.maxitems[WK_CONV], s);
+        const cudaError_t e = launch_small<false>(io, a, f, nprob, s);
         return e != cudaSuccess ? e : cudaGetLastError();
     }
-    const int nprob = a.count * a.nchan;
     cudaError_t e = optin_all(f);
     if (e != cudaSuccess) return e;
     RowIO r;

@@ -10,9 +10,7 @@ struct FFTArgs {
     int Nx, Ny;          // padded transform sizes (Nx even)
     int cpc;             // spectrum columns per CTA in the column pass
     int small;           // 1: one CTA per transform (Nx, Ny in 32 x {3, 4, 5});
-                         // hhat then lies in the order phase B reads it
-    int toy, tox;        // small: outputs of a tile
-    int one_tile;        // small: every stamp is one tile (the FFT method)
+                         // hhat then holds each column in warp-FFT order
     FFTPlan px, py;
     float2* tw_x;        // exp(-2 pi i k / Nx), k < Nx
     float2* tw_y;        // exp(-2 pi i k / Ny), k < Ny
@@ -54,11 +52,6 @@ struct RowInvIO {
 size_t fft_row_smem(int Nx);
 // the smallest 32 M >= n with M in {3, 4, 5} (the one-CTA transform), else 0
 int fft_small_len(int n);
-// the tiled method's transform side for a P x P PSF, and a tile's outputs along
-// y (multiples of 16) and x (multiples of 32, the trial partials' blocks)
-inline int fft_tile_len(int P) { return P <= 33 ? 96 : 128; }
-inline int fft_tile_toy(int P) { return (fft_tile_len(P) - P + 1) / 16 * 16; }
-inline int fft_tile_tox(int P) { return (fft_tile_len(P) - P + 1) / 32 * 32; }
 size_t fft_col_smem(int Ny, int cpc);
 cudaError_t launch_fft_twiddles(const FFTArgs& f, cudaStream_t s);
 cudaError_t launch_fft_psf(const FFTArgs& f, int count, const StampInfo* st, const float* psf,
