@@ -718,12 +718,10 @@ def run_batch(args):
         return n * len(sts) / (e0.elapsed_time(e1) / 1e3)
 
     # untimed setup: the direct convolution's launch shape tuned on these stamps
-    # (tile width per width class, tile height and persistent grid).  With 33 px
-    # PSFs the automatic method of a batched fit takes the one-CTA transform in
-    # tiles, which has no shape to tune: the two rates should agree.
+    # (tile width per width class, tile height and persistent grid), against
+    # the untuned cost model
     untuned = quick_rate()
-    d_direct = gf.make_desc(1, 1, s0.P, s0.kinds, s0.os_factor, 8, conv_method=gf.CONV_DIRECT)
-    gf.autotune(d_direct, batch, psf_d, ws=ws)
+    gf.autotune(d, batch, psf_d, ws=ws)
     tuned = quick_rate()
     shape = gf.conv_tile_shape(s0.P, 64)
     tiles = {int(c): gf.conv_tile_width(s0.P, 32 * int(c)) for c in sorted({(w + 31) // 32 for w in Ws})}
@@ -788,7 +786,7 @@ def run_batch(args):
             "data": "synthetic (seeded; true images rendered by the oracle)",
             "config": {"workload": "batch4096", "stamps": n,
                        "pixels": int(sum(h * w for h, w in zip(Hs, Ws))), "psf": s0.P,
-                       "conv": "auto: one-CTA transforms in overlap-save tiles",
+                       "conv": "auto: direct, tap rows summed apart",
                        "free_params": s0.nfree, "lm_tol": args.lm_tol,
                        "ladder": int(opts.ladder) or "auto",
                        "jacobian": args.jac,
@@ -803,8 +801,7 @@ def run_batch(args):
                     "h2d_bytes_per_step": int(img_p.numel() * 8 + psf_p.numel() * 4 + p0.size * 8),
                     "d2h_bytes_per_step": int(p0.size * 8 + n * 32)},
             "gpu_launches": launches,
-            "roofline": {"bound": "alu", "kernel": "k_conv_fft_small (5 N log2 N FLOP per length-N "
-                                                  "transform + 6 Ny per spectrum column)",
+            "roofline": {"bound": "alu", "kernel": "k_conv_direct (2 P^2 FLOP per output)",
                          "achieved": ach, "peak": fp32_peak, "unit": "TFLOP/s",
                          "frac": ach / fp32_peak, "traffic": None,
                          "peak_source": "measured FP32 FMA loop (gf_fma_peak) in this run",
@@ -1181,7 +1178,7 @@ def run_learned(args):
         f_hbm = gbs / hbm if hbm else None
         f_alu = ach / fp32_peak
         roof = {"bound": "hbm" if (f_hbm or 0) >= f_alu else "alu",
-                "kernel": f"k_conv_fft_small<{nx // 8},{ny // 8}> (one CTA per {ny} x {nx} "
+                "kernel": f"k_conv_fft_small<{nx // 32},{ny // 32}> (one CTA per {ny} x {nx} "
                           "transform of a stamp's channel)"}
         if roof["bound"] == "hbm":
             roof.update(achieved=gbs, peak=hbm, unit="GB/s", frac=f_hbm,

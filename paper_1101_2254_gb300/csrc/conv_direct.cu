@@ -631,7 +631,7 @@ cudaError_t launch_thin(const PassArgs& a, cudaStream_t s)
 //   P  9    7.6 /  9.8    7.7 /  9.8   7.7 /  9.7  11.0 / 11.9
 //   P 25   11.8 / 18.4   14.1 / 18.3  16.5 / 18.5  26.5 / 25.6
 //   P 33   16.1 / 24.5   20.5 / 24.5  24.6 / 24.5  40.9 / 36.4
-// PSFs above 35 px keep the generic kernel, which also multiplies its padding taps.
+// PSFs above 35 px keep k_conv_direct.
 long long conv_thin_max_blocks(int P) { return P > 35 ? 0 : (P < 33 ? 4 : 3) * 152; }
 
 template <bool ROWS>

@@ -298,7 +298,8 @@ __device__ void warp_bn(const Structure& S, WarpScratch& W, LMState* L)
     if (mine) v = PERT && part == 1 && analytic ? bn_deriv_lookup(n) : bn_lookup(n + v);
     // (An evaluation whose component has a NaN amplitude, as decoded from network
     // outputs outside the flux formula's domain, is NaN at every pixel whatever b_n:
-    // no solve.  8,192 starts of an untrained network, the launch: 632 us -> 53.)
+    // no solve.  8,192 starts of an untrained network, the launch: 632 us -> 53; a
+    // trained one's starts hardly have such components.)
     const bool unused = !PERT && !L && mine && isnan(amp_of(S, W.p, k));
     const unsigned miss = __ballot_sync(0xffffffffu, mine && isnan(v) && !unused);
     double* const vals = !PERT || part == 0 ? W.bn : analytic ? W.dbdn : W.bnp;
