@@ -56,11 +56,11 @@ TRAFFIC = {
     "stamp512": {
         # mean DRAM bytes per FFT launch of the fits (Jacobian and trial passes,
         # PSF spectra), from the capture in profiles/fft_traffic_stamp512.md
-        "bytes_per_launch": 1662083,
+        "bytes_per_launch": 1661495,
         "profile": "profiles/fft_traffic_stamp512.md",
         "sources": {
             "paper_1101_2254_gb300/csrc/conv_fft.cu":
-                "73ee748bbf63c92a06fc42eabd4aca15b7a5157dd557086529372e4065dc134e",
+                "82976b5b21fe1090dd5a26be77a9871e3808aefdd52f0fc28d2bda9f5ff141eb",
             "paper_1101_2254_gb300/csrc/conv_fft.cuh":
                 "a4d55cbdda7c2a8fcfe95457b1242aa8b387019fe6ead7c9f7ad84830167549d",
             "paper_1101_2254_gb300/csrc/fft.cuh":
@@ -79,11 +79,11 @@ TRAFFIC = {
 # once), so the bench scales it by the outputs of its average launch.  Null
 # once the kernel source differs from the one captured.
 CONV_DIRECT_TRAFFIC = {
-    # the 7-channel Jacobian launch of the profiled step (2352.2 MB read + 911.5 MB
-    # written); a fused trial launch moves 1219.6 MB for 2 rungs (18.2 B per output)
-    "bytes_per_output": 3.2637e9 / (7 * 8192 * 4096),
+    # the 7-channel Jacobian launch of the profiled step (2351.6 MB read + 914.9 MB
+    # written); a fused trial launch moves 626.7 MB for its rung (18.7 B per output)
+    "bytes_per_output": 3.2665e9 / (7 * 8192 * 4096),
     "profile": "profiles/k_conv_direct_learned8192.md",
-    "sources": {"paper_1101_2254_gb300/csrc/conv_direct.cu": "a0211dbd9cfc3e4a1c525d857c037a90f20008686be10873a8531cbb69679dfc"},
+    "sources": {"paper_1101_2254_gb300/csrc/conv_direct.cu": "9267c6d3a8154cd9b50630a47ec8d3a902a40e5f343e5d01e401015a5ba63219"},
 }
 
 
@@ -91,13 +91,13 @@ CONV_DIRECT_TRAFFIC = {
 # from the ncu capture of the Jacobian-pass launches on 8,192 stamps of the
 # learned workload; a launch's traffic grows in proportion to its transforms.
 CONV_FFT_SMALL_TRAFFIC = {
-    # the 7-channel Jacobian launch (57,344 transforms): 2423.4 MB read + 910.5 MB
-    # written = 58.1 KB per transform (the algorithmic grid + output: 53.2 KB)
-    "bytes_per_problem": (2423425792 + 910539520) / 57344,
+    # the 7-channel Jacobian launch (57,344 transforms): 2436.3 MB read + 914.8 MB
+    # written = 58.4 KB per transform (the algorithmic grid + output: 53.2 KB)
+    "bytes_per_problem": (2436304896 + 914819328) / 57344,
     "profile": "profiles/k_conv_fft_small_learned8192.md",
     "sources": {
         "paper_1101_2254_gb300/csrc/conv_fft.cu":
-            "73ee748bbf63c92a06fc42eabd4aca15b7a5157dd557086529372e4065dc134e",
+            "82976b5b21fe1090dd5a26be77a9871e3808aefdd52f0fc28d2bda9f5ff141eb",
         "paper_1101_2254_gb300/csrc/conv_fft.cuh":
             "a4d55cbdda7c2a8fcfe95457b1242aa8b387019fe6ead7c9f7ad84830167549d",
         "paper_1101_2254_gb300/csrc/warp_fft.cuh":
@@ -1197,8 +1197,10 @@ def run_learned(args):
                               "shared by its channels and not counted)",
             "hbm_gbs": gbs, "hbm_frac": f_hbm, "tflops": ach, "alu_frac": f_alu,
             "work_note": "5 N log2 N FLOP per length-N transform + 6 Ny per spectrum column",
-            "issue_note": "bound by latency: a barrier a phase and 24 warps an SM, 42 % of "
-                          "the issue rate at 21.7 thousand warp instructions a transform",
+            "issue_note": "bound by instruction issue: ncu measured smsp__issue_active at "
+                          "80.4 % of the issue rate on the Jacobian launch, the register "
+                          "FFT's shuffles and butterflies "
+                          "(profiles/k_conv_fft_small_learned8192.md)",
             "transforms": problems, "launches": pr["conv"]["launches"],
             "avg_launch_ms": conv_ms_avg,
             "share_of_device_time": pr["conv"]["ms"] / sum(v["ms"] for v in pr.values())})
@@ -1209,7 +1211,7 @@ def run_learned(args):
                 "traffic": conv_direct_traffic(conv_out / nconv),
                 "traffic_note": "bytes per launch: 13.9 B per output (ncu capture of "
                                 "the Jacobian launch, the dominant one; a fused trial "
-                                "launch moves 18.2 B per output; "
+                                "launch moves 18.7 B per output; "
                                 "profiles/k_conv_direct_learned8192.md) x the outputs "
                                 "of the average launch",
                 "alg_bytes_per_launch": 4.0 * (96 * 96 / 4096 + 1) * conv_out / nconv,
