@@ -348,18 +348,19 @@ __global__ void __launch_bounds__(WROW_WARPS * 32) k_fft_rows_inv_w(FFTArgs f, R
 // What bounds it is instruction issue.  Transforms in one thread's registers, with two
 // exchanges through shared memory, take half the instructions but a barrier a phase
 // at 24 warps an SM.  12 LM steps, us a step, these / those: one stamp of 64x64
-// 85 / 100, of 128x128 106 / 149, 16 of 128x128 152 / 202, 2,000 of 64x64 1,189 /
-// 1,271, 500 of 96x96 717 / 717, of 128x128 972 / 1,051.
+// 88 / 101, of 128x128 113 / 150, 16 of 128x128 149 / 202, 2,000 of 64x64 1,167 /
+// 1,265, 500 of 96x96 723 / 716, of 128x128 962 / 1,049.  Errors of the models of 35
+// stamps against 64 bits: 1.41e-7 / 1.30e-7.
 //
-// Warps a CTA: sixteen where shared memory holds one CTA an SM, 160 x 160 (with eight
-// the steps of 128x128 stamps above take 121, 168 and 1,115 us).
+// Warps a CTA: sixteen where shared memory holds one CTA an SM, 160 x 160 (for eight,
+// the steps of 128x128 stamps above: 121 -> 106, 168 -> 152 and 1,115 -> 972 us).
 constexpr int small_warps(int Nx, int Ny) { return Nx == 160 && Ny == 160 ? 16 : 8; }
 
 // Waves of CTAs a launch has at most.  One wave keeps its CTAs in step, all in the
 // same stage, and leaves SMs idle at its end; with a CTA for every stamp and channel, a
 // batch whose stamps have mostly left the loop launches thousands of them for
 // nothing.  8,192 fits of 64x64 stamps, convolution, ms, for one wave, four and a CTA
-// each: 15.9, 14.9, 17.2.
+// each (single stages, warp_fft.cuh): 15.9, 14.9, 17.2.
 constexpr int SMALL_WAVES = 4;
 
 struct SmallIO {
