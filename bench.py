@@ -60,13 +60,13 @@ TRAFFIC = {
         "profile": "profiles/fft_traffic_stamp512.md",
         "sources": {
             "paper_1101_2254_gb300/csrc/conv_fft.cu":
-                "82976b5b21fe1090dd5a26be77a9871e3808aefdd52f0fc28d2bda9f5ff141eb",
+                "d456d629860efb77a8ed55a3edf8db9c179fe1b090e8f343da4cae0df55f747d",
             "paper_1101_2254_gb300/csrc/conv_fft.cuh":
                 "a4d55cbdda7c2a8fcfe95457b1242aa8b387019fe6ead7c9f7ad84830167549d",
             "paper_1101_2254_gb300/csrc/fft.cuh":
                 "f12874458fbb0310b0b5f890cdc2b7d57b76b09e959613bf60669b0bcd060f50",
             "paper_1101_2254_gb300/csrc/warp_fft.cuh":
-                "968ef49fcdece8a3decab9e3bb9da728d116a1a103eff0d6437b5726e58de91b",
+                "f6cf3752396f815d4496b94ec0a1610320ba7c965a39c3d9f1e39eb373bebe0a",
         },
     },
 }
@@ -91,17 +91,17 @@ CONV_DIRECT_TRAFFIC = {
 # from the ncu capture of the Jacobian-pass launches on 8,192 stamps of the
 # learned workload; a launch's traffic grows in proportion to its transforms.
 CONV_FFT_SMALL_TRAFFIC = {
-    # the 7-channel Jacobian launch (57,344 transforms): 2436.3 MB read + 914.8 MB
+    # the 7-channel Jacobian launch (57,344 transforms): 2435.8 MB read + 914.6 MB
     # written = 58.4 KB per transform (the algorithmic grid + output: 53.2 KB)
-    "bytes_per_problem": (2436304896 + 914819328) / 57344,
+    "bytes_per_problem": (2435835136 + 914584576) / 57344,
     "profile": "profiles/k_conv_fft_small_learned8192.md",
     "sources": {
         "paper_1101_2254_gb300/csrc/conv_fft.cu":
-            "82976b5b21fe1090dd5a26be77a9871e3808aefdd52f0fc28d2bda9f5ff141eb",
+            "d456d629860efb77a8ed55a3edf8db9c179fe1b090e8f343da4cae0df55f747d",
         "paper_1101_2254_gb300/csrc/conv_fft.cuh":
             "a4d55cbdda7c2a8fcfe95457b1242aa8b387019fe6ead7c9f7ad84830167549d",
         "paper_1101_2254_gb300/csrc/warp_fft.cuh":
-            "968ef49fcdece8a3decab9e3bb9da728d116a1a103eff0d6437b5726e58de91b",
+            "f6cf3752396f815d4496b94ec0a1610320ba7c965a39c3d9f1e39eb373bebe0a",
         "paper_1101_2254_gb300/csrc/fft.cuh":
             "f12874458fbb0310b0b5f890cdc2b7d57b76b09e959613bf60669b0bcd060f50",
     },
@@ -1198,7 +1198,7 @@ def run_learned(args):
             "hbm_gbs": gbs, "hbm_frac": f_hbm, "tflops": ach, "alu_frac": f_alu,
             "work_note": "5 N log2 N FLOP per length-N transform + 6 Ny per spectrum column",
             "issue_note": "bound by instruction issue: ncu measured smsp__issue_active at "
-                          "80.4 % of the issue rate on the Jacobian launch, the register "
+                          "78.2 % of the issue rate on the Jacobian launch, the register "
                           "FFT's shuffles and butterflies "
                           "(profiles/k_conv_fft_small_learned8192.md)",
             "transforms": problems, "launches": pr["conv"]["launches"],

@@ -139,10 +139,10 @@ __device__ __forceinline__ int bitrev5(int l) { return (int)(__brev((unsigned)l)
 // 1996): in each pair (d, d / 2) both butterflies are a = p + sg v (sg = -1 on the
 // upper lane, +1 on the lower), the factor between them is i or 1, so a swap, and one
 // product by w_2d^{(l mod d / 2) q}, q = bit d of l + 2 bit d / 2, follows the second.  Two
-// products instead of the four of single stages: 11 % fewer instructions, and fewer
-// roundings, of the twiddles above all, whose magnitudes' errors add up over a forward and
-// an inverse transform (error of a 96 x 96 convolution of a galaxy, norm against 64 bits:
-// 1.9e-7 -> 1.7e-7, restated in numpy; in-register transforms, conv_fft.cu: 1.2e-7).
+// products instead of the four of single stages: 7 % fewer instructions in a 96 x 96
+// convolution (39.3 -> 36.6 thousand a transform), and fewer roundings, of the
+// twiddles above all, whose magnitudes' errors add up over a forward and an inverse
+// transform (models of 35 stamps, norm against 64 bits: 1.51e-7 -> 1.41e-7).
 template <int M>
 struct WarpTw {
     float2 rm[M];  // e^{-2 pi i k / M}
