@@ -133,7 +133,7 @@ typedef enum {
                            (For extended grids up to 160 x 160 the FFT is one CTA per
                            transform and overtakes the direct sum from about P = 15 on
                            64x64 and 96x96 stamps, P = 33 on 32x32: name GF_CONV_FFT
-                           there, if round-off of 2e-7 of the brightest pixel in every
+                           there, if round-off of 2e-7 to 5e-7 of the brightest in every
                            pixel will do: on a faint sky beside a bright compact source
                            that can be a hundredth of the pixel.) */
     GF_CONV_DIRECT = 1, /* tiled direct sum, PSF and halo tile in shared memory; the P^2
